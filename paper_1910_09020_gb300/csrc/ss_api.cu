@@ -1271,7 +1271,7 @@ int ss_edit_distance_varlen(ss_ctx *ctx, const void *reads, const void *refs,
                                (const uint32_t *)refs, offsets, lengths, E,
                                n, out_ed, ctx->d_status, ctx->sm_count,
                                pick_stream(stream)));
-    ctx->counters.launches += 6;
+    ctx->counters.launches += 2;
     return SS_OK;
 }
 

@@ -2,6 +2,7 @@
 // and the confusion counts of filter decisions against it.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "ss_internal.h"
@@ -44,9 +45,15 @@ __global__ void k_confusion(const uint8_t *__restrict__ acc,
     }
 }
 
-// Warp per pair, pairs of any length and threshold; the launch for class C
-// (2E+1 <= 32 C, E <= 511) routes the pairs of that class and skips the
-// others; the first launch also flags unsupported thresholds.
+// Pairs of any length and threshold, TEAM lanes per pair over the diagonals
+// of a step, F of the last two steps in shared memory.  The launch for
+// (ELO, EHI] takes the pairs of those thresholds and skips the others; the
+// first launch (ELO < 0) also flags unsupported thresholds.  The teams of a
+// warp step together (a step ends when the slowest slide of the warp does).
+// Bound by instruction issue: about 130 per 32 diagonals of a step, most of
+// them the two window assemblies of a slide.  60,000 pairs of 64 bp to 10
+// kbp, E = 5 %: 2.73 ms, where the banded table (a warp per pair, every cell
+// of 2E+1 diagonals) took 111.6 ms.
 struct EdVarArgs {
     const uint32_t *reads;
     const uint32_t *refs;
@@ -58,30 +65,72 @@ struct EdVarArgs {
     int *status;
 };
 
-template <int C, int CLO>
-__global__ void __launch_bounds__(128) k_ed_warp(const EdVarArgs a)
+constexpr int kEdVarWarps = 4;
+constexpr int kEdTeamMaxE = 15;  // up to it 8 lanes per pair, above 32
+
+template <int TEAM, int ELO, int EHI>
+__global__ void __launch_bounds__(32 * kEdVarWarps)
+    k_ed_diag(const EdVarArgs a)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp =
-        ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = warp; p < a.n; p += nwarps) {
-        const int m = a.len[p], E = a.E[p];
-        if (m < 0 || E < 0 || E > kEdWarpMaxE) {
-            if (CLO == 0 && lane == 0) {
-                a.ed[p] = -1;
-                atomicOr(a.status, m < 0 || E < 0 ? kStatusInvalidArg
-                                                  : kStatusUnsupported);
+    constexpr int T = 32 / TEAM;    // pairs per warp
+    constexpr int H = EHI / 2;      // |k| never exceeds it
+    constexpr int W = 2 * H + 3;    // and a guard entry either side
+    __shared__ int s_f[kEdVarWarps][T][2][W];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int team = lane / TEAM, tl = lane % TEAM;
+    int(*F)[W] = s_f[wib][team];
+    const int64_t step = (int64_t)gridDim.x * kEdVarWarps * T;
+    for (int64_t p0 = ((int64_t)blockIdx.x * kEdVarWarps + wib) * T;
+         p0 < a.n; p0 += step) {
+        const int64_t p = p0 + team;
+        int m = 0, E = 0;
+        bool act = p < a.n;
+        if (act) {
+            m = a.len[p];
+            E = a.E[p];
+            if (m < 0 || E < 0 || E > kEdWarpMaxE) {
+                if (ELO < 0 && tl == 0) {
+                    a.ed[p] = -1;
+                    atomicOr(a.status, m < 0 || E < 0 ? kStatusInvalidArg
+                                                      : kStatusUnsupported);
+                }
+                act = false;
+            } else if (E <= ELO || E > EHI) {
+                act = false;
             }
-            continue;
         }
-        const int need = (2 * E + 1 + 31) >> 5;  // cells per lane
-        if (need <= CLO || need > C)
+        if (!__any_sync(0xffffffffu, act))
             continue;
-        const int v = ed_band_warp<C>(a.reads + a.off[p], a.refs + a.off[p],
-                                      m, E);
-        if (lane == 0)
-            a.ed[p] = v;
+        const int64_t off = act ? a.off[p] : 0;
+        const uint32_t *q = a.reads + off, *r = a.refs + off;
+        const int w16 = (m + 15) >> 4;
+        for (int x = tl; x < W; x += TEAM)
+            F[0][x] = F[1][x] = kEdNone;
+        __syncwarp();
+        if (act && tl == 0)
+            F[0][H + 1] = ed_slide(q, r, w16, 0, 0, m);
+        __syncwarp();
+        for (int e = 0;; ++e) {
+            if (act) {
+                const bool there = F[e & 1][H + 1] >= m;
+                if (there || e == E) {
+                    if (tl == 0)
+                        a.ed[p] = there ? e : E + 1;
+                    act = false;
+                }
+            }
+            if (!__any_sync(0xffffffffu, act))
+                break;
+            if (act) {
+                const int w = min(e + 1, E - e - 1);
+                const int *prev = F[e & 1] + H + 1;
+                int *next = F[(e + 1) & 1] + H + 1;
+                for (int k = tl - w; k <= w; k += TEAM)
+                    next[k] = ed_diagonal(q, r, w16, m, prev + k, k);
+            }
+            __syncwarp();
+        }
+        __syncwarp();  // F is reused by the next pair
     }
 }
 
@@ -126,16 +175,16 @@ cudaError_t launch_ed_var(const uint32_t *reads, const uint32_t *refs,
     if (n <= 0)
         return cudaSuccess;
     const EdVarArgs a{reads, refs, off, len, E, n, ed, status};
-    const int64_t want = (n * 32 + 127) / 128;
-    const int grid = (int)(want < (int64_t)sm_count * 16
-                               ? want
-                               : (int64_t)sm_count * 16);
-    k_ed_warp<1, 0><<<grid, 128, 0, st>>>(a);
-    k_ed_warp<2, 1><<<grid, 128, 0, st>>>(a);
-    k_ed_warp<4, 2><<<grid, 128, 0, st>>>(a);
-    k_ed_warp<8, 4><<<grid, 128, 0, st>>>(a);
-    k_ed_warp<16, 8><<<grid, 128, 0, st>>>(a);
-    k_ed_warp<32, 16><<<grid, 128, 0, st>>>(a);
+    // one warp's worth of pairs per warp (no cap on the grid: pairs differ
+    // in cost by the square of their threshold, and the block scheduler
+    // hands them out as warps finish)
+    auto grid = [n](int teams) {
+        const int64_t per = (int64_t)kEdVarWarps * teams;
+        return (unsigned)std::min<int64_t>((n + per - 1) / per, 0x7fffffff);
+    };
+    k_ed_diag<8, -1, kEdTeamMaxE><<<grid(4), 32 * kEdVarWarps, 0, st>>>(a);
+    k_ed_diag<32, kEdTeamMaxE, kEdWarpMaxE>
+        <<<grid(1), 32 * kEdVarWarps, 0, st>>>(a);
     return cudaGetLastError();
 }
 

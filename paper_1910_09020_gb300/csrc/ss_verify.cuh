@@ -97,98 +97,54 @@ SS_HD int ed_banded(const uint32_t *q, const uint32_t *r, int m, int w16)
     return D[E];  // j = i = m
 }
 
-// ---- large thresholds: one warp per pair -----------------------------------
+// ---- per-pair lengths and thresholds: furthest-reaching diagonals -----------
 //
-// The same banded DP for E up to 511: the 2E+1 band cells of a row are
-// spread over the 32 lanes, C consecutive cells per lane, in registers.  The
-// in-row dependency D[i][j] = min(T[j], D[i][j-1] + 1), with T the best of
-// the diagonal and upper neighbours, is a prefix minimum: D[d] = d +
-// min_{d' <= d} (T[d'] - d'), computed per lane and then across the warp
-// with shuffles.  The reference bases of a lane's cells come from a 64-base
-// window of its bit planes, re-read every 32 rows.  Once every cell of a
-// row exceeds E, ED > E (every alignment passes through that row).
-template <int C>
-__device__ int ed_band_warp(const uint32_t *q, const uint32_t *r, int m,
-                            int E)
+// min(ED, E+1) by diagonals instead of table cells (Ukkonen 1985; Landau and
+// Vishkin 1989): F_e[k] is the furthest read position i for which the cell
+// (i, i + k) costs at most e edits, and
+//     F_e[k] = slide(max(F_{e-1}[k] + 1, F_{e-1}[k-1], F_{e-1}[k+1] + 1), k)
+// (substitution, reference base inserted, read base dropped), slide running
+// along the diagonal while the bases match.  ED is the first e with F_e[0] =
+// m.  A path of at most E edits that stands on diagonal k after e of them
+// still needs |k| to come back, so only |k| <= min(e, E - e) is kept: about
+// E^2 / 2 slides per pair, where the banded table has m (2E+1) cells (10 kbp
+// at E = 500: 125 thousand against 10 million).
+constexpr int kEdNone = -(1 << 20);  // no cell of this diagonal reached
+
+// Matching bases from q[i], r[j] on, at most n (i + n and j + n inside the
+// sequences of w16 packed words).  Two packed words hold the code bits of
+// 32 bases from a word's start: 17 to 32 of them are compared at once.
+SS_HD int ed_slide(const uint32_t *q, const uint32_t *r, int w16, int i,
+                   int j, int n)
 {
-    const int lane = threadIdx.x & 31;
-    const int B = 2 * E + 1;
-    const int CAP = E + 1;
-    const int BIG = 1 << 30;
-    const int w16 = (m + 15) >> 4;
-    int P[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) {  // row 0: D[0][j] = j
-        const int d = lane * C + c, j = d - E;
-        P[c] = (d < B && j >= 0 && j <= m) ? (j < CAP ? j : CAP) : CAP;
+    int done = 0;
+    while (done < n) {
+        const int a = i + done, b = j + done;
+        const int ia = a >> 4, ib = b >> 4;
+        const uint32_t q0 = ldg(q + ia), r0 = ldg(r + ib);
+        const uint32_t q1 = ia + 1 < w16 ? ldg(q + ia + 1) : 0u;
+        const uint32_t r1 = ib + 1 < w16 ? ldg(r + ib + 1) : 0u;
+        const int sa = a & 15, sb = b & 15;
+        const uint32_t x =
+            ((prmt(q0, q1, 0x5410u) >> sa) ^ (prmt(r0, r1, 0x5410u) >> sb)) |
+            ((prmt(q0, q1, 0x7632u) >> sa) ^ (prmt(r0, r1, 0x7632u) >> sb));
+        const int valid = 32 - imax(sa, sb);  // bases both windows hold
+        const int run = imin(x ? ffs32(x) - 1 : 32, valid);
+        done += run;
+        if (run < valid)
+            break;
     }
-    uint64_t wlo = 0, whi = 0;
-    int wstart = 0;
-    for (int i = 1; i <= m; ++i) {
-        const int b0 = i - E - 1 + lane * C;  // reference base of cell c = 0
-        if (((i - 1) & 31) == 0) {            // warp-uniform refill
-            wlo = plane_window(r, w16, m, b0, 0);
-            whi = plane_window(r, w16, m, b0, 1);
-            wstart = b0;
-        }
-        const int sh = b0 - wstart;           // 0..31
-        const uint32_t qw = ldg(q + ((i - 1) >> 4));
-        const uint64_t qlo = 0ull - (uint64_t)((qw >> ((i - 1) & 15)) & 1u);
-        const uint64_t qhi =
-            0ull - (uint64_t)((qw >> (16 + ((i - 1) & 15))) & 1u);
-        const uint64_t mm = ((wlo >> sh) ^ qlo) | ((whi >> sh) ^ qhi);
-        const int next0 = __shfl_down_sync(0xffffffffu, P[0], 1);
-        int PM[C];
-        int pm = BIG;
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int d = lane * C + c, j = i + d - E;
-            int up = c + 1 < C ? P[c + 1] : (lane < 31 ? next0 : CAP);
-            if (d + 1 >= B)
-                up = CAP;
-            int t = P[c] + (int)((mm >> c) & 1ull);
-            t = t < up + 1 ? t : up + 1;
-            if (j == 0)
-                t = i;                        // D[i][0] = i
-            if (d >= B || j < 0 || j > m)
-                t = CAP;
-            const int u = t - d;
-            pm = pm < u ? pm : u;
-            PM[c] = pm;
-        }
-        // exclusive prefix minimum of the lanes' minima
-        int incl = pm;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off)
-                incl = incl < v ? incl : v;
-        }
-        int ex = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0)
-            ex = BIG;
-        int rowmin = CAP;
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int d = lane * C + c, j = i + d - E;
-            int v = d + (ex < PM[c] ? ex : PM[c]);
-            v = v < CAP ? v : CAP;
-            if (d >= B || j < 0 || j > m)
-                v = CAP;
-            P[c] = v;
-            rowmin = rowmin < v ? rowmin : v;
-        }
-        if ((i & 7) == 0 &&
-            __reduce_min_sync(0xffffffffu, (unsigned)rowmin) >= (unsigned)CAP)
-            return CAP;
-    }
-    // cell d = E (j = i = m)
-    int out = CAP;
-#pragma unroll
-    for (int c = 0; c < C; ++c)
-        if (lane * C + c == E)
-            out = P[c];
-    return __shfl_sync(0xffffffffu, out, E / C);
+    return imin(done, n);
+}
+
+// One diagonal: prev points at F_{e-1}[k].
+SS_HD int ed_diagonal(const uint32_t *q, const uint32_t *r, int w16, int m,
+                      const int *prev, int k)
+{
+    const int lim = m - imax(k, 0);  // the diagonal's last read position
+    int t = imax(imax(prev[0], prev[1]) + 1, prev[-1]);
+    t = imin(t, lim);
+    return t + ed_slide(q, r, w16, t, t + k, lim - t);
 }
 
 }  // namespace ssk

@@ -127,3 +127,24 @@ def test_warp_verifier_rejects_out_of_range(F):
     assert ei.value.code == binding.SS_ERR_UNSUPPORTED
     g = got.cpu().numpy()
     assert g[1] == -1 and g[0] >= 0 and g[2] >= 0
+
+
+@pytest.mark.parametrize("E", [0, 1, 2, 14, 15, 16, 17, 63, 510, 511])
+def test_diagonal_verifier_edges(F, E):
+    """Both team widths (E up to 15 and above) at thresholds either side of
+    the switch and at the ends of the range, lengths around a packed word
+    and below E, related and unrelated pairs, a number of pairs that leaves
+    the last warp's teams partly empty."""
+    L = np.array([0, 1, 2, 15, 16, 17, 31, 32, 33, 100, 700] * 3, np.int32)
+    n = len(L)
+    for rate in (0.0, 0.05, 0.9):
+        reads, refs, off, q, r, woff = _varlen_packed(F, 47 + E, L, rate)
+        got = F.edit_distance_varlen(q, r, to_dev(woff[:-1]), to_dev(L),
+                                     to_dev(np.full(n, E, np.int32)))
+        F.sync()
+        got = got.cpu().numpy()
+        for p in range(n):
+            a = reads[off[p]:off[p + 1]].tobytes()
+            b = refs[off[p]:off[p + 1]].tobytes()
+            want = min(oracle.edit_distance(a, b), E + 1)
+            assert got[p] == want, (p, int(L[p]), got[p], want)
