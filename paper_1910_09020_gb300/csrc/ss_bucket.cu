@@ -24,6 +24,8 @@
 
 #include "ss_bucket.cuh"
 #include "ss_cw.cuh"
+#include "ss_cwt.cuh"
+#include "ss_cwx.cuh"
 #include "ss_device.cuh"
 #include "ss_internal.h"
 #include "ss_rw.cuh"
@@ -116,8 +118,8 @@ __global__ void __launch_bounds__(kRwThreads)
     }
 }
 
-// Serving: put the pairs of the CTA-per-pair classes that the long-pair
-// queue takes into its ring (one thread per pair; an entry is published
+// Serving: put the pairs of the classes that the long-pair queue takes into
+// its ring (one thread per pair; an entry is published
 // by its seq, written after the entry's other fields).  The batch's
 // descriptor already holds how many there are (the host counts them with
 // the same rule); a different count here latches kStatusUnsupported.
@@ -130,13 +132,10 @@ __global__ void __launch_bounds__(256)
         s_n = 0;
     __syncthreads();
     int mine = 0;
-    for (int cls = kRwClasses + kCwwClasses; cls < kClasses; ++cls) {
+    for (int cls = kFirstIndex; cls < kFirstCta; ++cls) {
         const int begin = ws.ranges[2 * cls], end = ws.ranges[2 * cls + 1];
         for (int i = begin + (int)threadIdx.x; i < end; i += blockDim.x) {
             const int64_t p = ws.perm[i];
-            const int m = ps.len(p);
-            if (!long_queued(cls, m, eff_threshold(m, ps.thr(p))))
-                continue;
             const unsigned long long pos = atomicAdd(h.q.tail, 1ull);
             LongEntry *e = h.q.ring + (pos & (kLongRing - 1));
             e->pair = p;
@@ -219,19 +218,24 @@ BucketWs bucket_ws_at(void *base, int64_t n)
 // Bytes cleared at the start of every pass (hist and ndeferred).
 static size_t bucket_clear_bytes() { return (size_t)kKeys * 4 + 16; }
 
-// Largest staged pair (in shared words) of each column-wise class.
-int cw_class_slice_words(int cls)
+// Shared memory of a CTA of each team, index and CTA class: its pairs' (the
+// longest the class takes) staged words or tables.
+size_t cw_class_smem(int cls)
 {
-    if (cls >= kRwClasses && cls < kRwClasses + kCwwClasses) {
-        const int Mb = cww_mbound(cls - kRwClasses);
-        return CwLayout::of(Mb, kCwwMaxE).words();
+    if (cls < kFirstIndex) {
+        const int c = cls - kFirstTeam;
+        const int pairs = kTeamWarps * 32 / team_lanes(team_width_of(c));
+        return (size_t)pairs * TeamLayout::of(team_mbound(c)).words() * 4;
     }
-    const int i = cls - kRwClasses - kCwwClasses;
-    const int w = i / kCwcMbounds, b = i % kCwcMbounds;
-    const int Mb = cwc_mbound(b);
-    int Emax = w == kCwcWidths - 1 ? Mb - 1 : (32 * cwc_width(w) - 1) / 2;
-    Emax = std::min(Emax, Mb - 1);
-    return CwLayout::of(Mb, Emax).words();
+    switch (cls - kFirstIndex) {
+    case 0: return IndexShape0::WORDS * 4;
+    case 1: return IndexShape1::WORDS * 4;
+    case 2: return IndexShape2::WORDS * 4;
+    case 3: return IndexShape3::WORDS * 4;
+    default: break;
+    }
+    const int M = cta_mbound(cls - kFirstCta);
+    return (size_t)CwLayout::of(M, M - 1).words() * 4;
 }
 
 namespace {
@@ -257,8 +261,7 @@ int occupancy_per_sm(KernelT kernel, int threads, size_t smem)
 // by side.  Written once under g_init_mu before `ready` is released; read
 // only by threads that saw it set.
 struct LaunchCfg {
-    int rw[kRwClasses];
-    int cw[3][kClasses];  // [subgrid 4/8/16][class]
+    int per_sm[kClasses];      // the CTA classes' at subgrid 8
     std::atomic<bool> ready{false};
 };
 LaunchCfg g_cfg[kMaxDevices];
@@ -278,32 +281,29 @@ const LaunchCfg *launch_cfg()
     return &g_cfg[d];
 }
 
-int kidx(int k) { return k == 4 ? 0 : k == 16 ? 2 : 1; }
+using CwKernel = void (*)(CwArgs);
 
-template <int K>
-cudaError_t init_cw(LaunchCfg &cfg)
+// Kernel and CTA width of a team, index or (subgrid k) CTA class.
+CwKernel cw_kernel(int cls, int k, unsigned &threads)
 {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_cw_warp<K>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_cw_cta<K>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024)) != cudaSuccess)
-        return e;
-    for (int c = 0; c < kCwwClasses; ++c) {
-        const int cls = kRwClasses + c;
-        const size_t smem = (size_t)4 * cw_class_slice_words(cls) * 4;
-        cfg.cw[kidx(K)][cls] = occupancy_per_sm(k_cw_warp<K>, 128, smem);
-    }
-    for (int w = 0; w < kCwcWidths; ++w)
-        for (int b = 0; b < kCwcMbounds; ++b) {
-            const int cls = cwc_class(w, b);
-            const size_t smem = (size_t)cw_class_slice_words(cls) * 4;
-            cfg.cw[kidx(K)][cls] =
-                occupancy_per_sm(k_cw_cta<K>, cwc_width(w), smem);
+    if (cls < kFirstIndex) {
+        threads = 32 * kTeamWarps;
+        switch (team_width_of(cls - kFirstTeam)) {
+        case 0: return k_cw_team<team_lanes(0)>;
+        case 1: return k_cw_team<team_lanes(1)>;
+        default: return k_cw_team<team_lanes(2)>;
         }
-    return cudaSuccess;
+    }
+    threads = kIndexThreads;
+    switch (cls - kFirstIndex) {
+    case 0: return k_cw_index<0>;
+    case 1: return k_cw_index<1>;
+    case 2: return k_cw_index<2>;
+    case 3: return k_cw_index<3>;
+    default: break;
+    }
+    threads = kCtaThreads;
+    return k == 4 ? k_cw_cta<4> : k == 16 ? k_cw_cta<16> : k_cw_cta<8>;
 }
 
 }  // namespace
@@ -322,15 +322,22 @@ cudaError_t bucket_init()
         return cudaSuccess;
     if ((e = rw_init(d)) != cudaSuccess)
         return e;
-    cfg.rw[0] = occupancy_per_sm(k_rw_bucket<1>, 128, 0);
-    cfg.rw[1] = occupancy_per_sm(k_rw_bucket<3>, 128, 0);
-    cfg.rw[2] = occupancy_per_sm(k_rw_bucket<7>, 128, 0);
-    cfg.rw[3] = occupancy_per_sm(k_rw_bucket<15>, 128, 0);
-    cfg.rw[4] = occupancy_per_sm(k_rw_bucket<31>, 128, 0);
-    if ((e = init_cw<4>(cfg)) != cudaSuccess ||
-        (e = init_cw<8>(cfg)) != cudaSuccess ||
-        (e = init_cw<16>(cfg)) != cudaSuccess)
-        return e;
+    cfg.per_sm[0] = occupancy_per_sm(k_rw_bucket<1>, 128, 0);
+    cfg.per_sm[1] = occupancy_per_sm(k_rw_bucket<3>, 128, 0);
+    cfg.per_sm[2] = occupancy_per_sm(k_rw_bucket<7>, 128, 0);
+    cfg.per_sm[3] = occupancy_per_sm(k_rw_bucket<15>, 128, 0);
+    cfg.per_sm[4] = occupancy_per_sm(k_rw_bucket<31>, 128, 0);
+    for (int k : {4, 16, 8})
+        for (int cls = kFirstTeam; cls < kClasses; ++cls) {
+            unsigned threads = 0;
+            const CwKernel f = cw_kernel(cls, k, threads);
+            if ((e = cudaFuncSetAttribute(
+                     f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                     200 * 1024)) != cudaSuccess)
+                return e;
+            cfg.per_sm[cls] =
+                occupancy_per_sm(f, (int)threads, cw_class_smem(cls));
+        }
     cfg.ready.store(true, std::memory_order_release);
     return cudaSuccess;
 }
@@ -453,36 +460,30 @@ cudaError_t launch_if(const ScanCond &c, Fan *fan, int h,
 
 // counts (may be null): an upper bound of each class's pairs known on the
 // host; classes it bounds by 0 are not launched.
-template <int K>
-cudaError_t launch_cw_classes(const LaunchCfg &cfg, CwArgs a, int sm_share,
-                              const ScanCond &c, Fan *fan, cudaStream_t st,
-                              const int64_t *counts)
+cudaError_t launch_cw_classes(const LaunchCfg &cfg, CwArgs a, int subgrid,
+                              int sm_share, const ScanCond &c, Fan *fan,
+                              cudaStream_t st, const int64_t *counts)
 {
-    cudaError_t e;
-    for (int k = 0; k < kCwwClasses; ++k) {
-        a.cls = kRwClasses + k;
+    // the index classes first: the pairs that take longest from start to end
+    for (int i = 0; i < kClasses - kFirstTeam; ++i) {
+        a.cls = i < kClasses - kFirstIndex ? kFirstIndex + i
+                                           : kFirstTeam + i -
+                                                 (kClasses - kFirstIndex);
         if (counts && counts[a.cls] == 0)
             continue;
-        a.slice_words = cw_class_slice_words(a.cls);
-        const size_t smem = (size_t)4 * a.slice_words * 4;
-        if ((e = launch_if(c, fan, a.cls, k_cw_warp<K>,
-                           (unsigned)(cfg.cw[kidx(K)][a.cls] * sm_share), 128,
-                           smem, st, a)) != cudaSuccess)
+        a.slice_words = a.cls < kFirstIndex
+                            ? TeamLayout::of(team_mbound(a.cls - kFirstTeam))
+                                  .words()
+                            : 0;
+        unsigned threads = 0;
+        const CwKernel f = cw_kernel(a.cls, subgrid, threads);
+        const cudaError_t e =
+            launch_if(c, fan, a.cls, f,
+                      (unsigned)(cfg.per_sm[a.cls] * sm_share), threads,
+                      cw_class_smem(a.cls), st, a);
+        if (e != cudaSuccess)
             return e;
     }
-    for (int w = 0; w < kCwcWidths; ++w)
-        for (int b = 0; b < kCwcMbounds; ++b) {
-            a.cls = cwc_class(w, b);
-            if (counts && counts[a.cls] == 0)
-                continue;
-            a.slice_words = cw_class_slice_words(a.cls);
-            const size_t smem = (size_t)a.slice_words * 4;
-            if ((e = launch_if(c, fan, a.cls, k_cw_cta<K>,
-                               (unsigned)(cfg.cw[kidx(K)][a.cls] * sm_share),
-                               (unsigned)cwc_width(w), smem, st, a)) !=
-                cudaSuccess)
-                return e;
-        }
     return cudaSuccess;
 }
 
@@ -499,7 +500,7 @@ cudaError_t launch_rw_classes(const LaunchCfg &cfg, CwArgs a, int sm_share,
         if (counts && counts[k] == 0)
             continue;
         const cudaError_t e =
-            launch_if(c, fan, k, kern[k], (unsigned)(cfg.rw[k] * sm_share),
+            launch_if(c, fan, k, kern[k], (unsigned)(cfg.per_sm[k] * sm_share),
                       128, 0, st, a);
         if (e != cudaSuccess)
             return e;
@@ -577,7 +578,7 @@ cudaError_t launch_bucketed(const PairSet &ps, const BucketWs &ws,
     const int sh = sm_count;  // persistent grids span this many SMs
     CwArgs a{ps, ws, 0, 0};
     if (hook) {
-        // serving: the queue's share of the CTA-per-pair classes
+        // serving: the pairs the queue takes
         k_long_enqueue<<<1, 256, 0, st>>>(ps, ws, *hook, hook_expect, status);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
@@ -591,7 +592,7 @@ cudaError_t launch_bucketed(const PairSet &ps, const BucketWs &ws,
         if ((e = fan_begin(fan, st)) != cudaSuccess)
             return e;
     } else {
-        // direct: column-wise classes on the side stream
+        // direct: the classes above E' = 31 on the side stream
         if ((e = cudaEventRecord(fork, st)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess)
             return e;
@@ -600,11 +601,7 @@ cudaError_t launch_bucketed(const PairSet &ps, const BucketWs &ws,
     const int64_t *cc = class_counts;
     if ((e = launch_rw_classes(*cfg, a, sh, c, &fan, st, cc)) != cudaSuccess)
         return e;
-    switch (tp.cw_subgrid) {
-    case 4: e = launch_cw_classes<4>(*cfg, a, sh, c, &fan, cw_st, cc); break;
-    case 16: e = launch_cw_classes<16>(*cfg, a, sh, c, &fan, cw_st, cc); break;
-    default: e = launch_cw_classes<8>(*cfg, a, sh, c, &fan, cw_st, cc); break;
-    }
+    e = launch_cw_classes(*cfg, a, tp.cw_subgrid, sh, c, &fan, cw_st, cc);
     if (e != cudaSuccess)
         return e;
     *launches += kClasses + 1;
@@ -643,7 +640,8 @@ cudaError_t launch_bucketed_one_stream(const PairSet &ps, const BucketWs &ws,
     if ((e = launch_rw_classes(*cfg, a, sm_count, c, nullptr, st,
                                nullptr)) != cudaSuccess)
         return e;
-    return launch_cw_classes<8>(*cfg, a, sm_count, c, nullptr, st, nullptr);
+    return launch_cw_classes(*cfg, a, tp.cw_subgrid, sm_count, c, nullptr, st,
+                             nullptr);
 }
 
 }  // namespace ssk

@@ -5,9 +5,11 @@
 // length m and effective threshold E' = min(E, m-1) (rows with |s| >= m hold
 // no Q base at all, so they are all obstacles and never bound the longest
 // run; the count limit still uses E):
-//   * RW  classes: E' <= 31, thread per pair, E' <= EMAX in {1, 3, 7, 15, 31}
-//   * CWW classes: 32 <= E' <= 511 and m <= 16384, warp per pair, by m bound
-//   * CWC classes: larger, CTA per pair, by CTA width and m bound
+//   * RW classes: E' <= 31, thread per pair, E' <= EMAX in {1, 3, 7, 15, 31}
+//   * team classes: 32 <= E' <= 496 and m <= 16384, 8, 16 or 32 lanes per
+//     pair (ss_cwt.cuh), by team width and m bound
+//   * index classes: E' <= 10016, CTA per pair (ss_cwx.cuh), by E'
+//   * CTA classes: larger E', CTA per pair (ss_cw.cuh), by m bound
 // Within a class pairs are ordered by length, longest first (quarter-octave
 // bins), so that persistent workers take the biggest pairs first and a warp
 // of the RW kernel sees similar lengths.
@@ -23,25 +25,46 @@ __host__ __device__ constexpr int rw_emax(int c)
 {
     return c == 0 ? 1 : c == 1 ? 3 : c == 2 ? 7 : c == 3 ? 15 : 31;
 }
-// m bounds of the warp-per-pair classes: a class's shared-memory slice is
-// sized for its bound, so finer bounds put more CTAs on an SM (the kernel
-// is latency-bound; its shared memory sets the CTAs per SM from 6 KB on)
-constexpr int kCwwClasses = 7;
-__host__ __device__ constexpr int cww_mbound(int c)
+// Team classes.  A team's lanes each take one aligned word of 32 starts, and
+// 2E+1 starts touch at most (2E + 31) / 32 + 1 words (rounded down), so
+// teams of 8, 16 and 32 lanes cover a pair up to E' = 112, 240 and 496.  A class's shared-memory slice is sized for its m bound, so
+// finer bounds put more pairs on an SM.
+constexpr int kTeamWidths = 3;
+__host__ __device__ constexpr int team_lanes(int w) { return 8 << w; }
+__host__ __device__ constexpr int team_max_e(int w)
 {
-    return c == 0 ? 2048 : c == 1 ? 3072 : c == 2 ? 4096 : c == 3 ? 6144
-         : c == 4 ? 8192 : c == 5 ? 12288 : 16384;
+    return w == 0 ? 112 : w == 1 ? 240 : 496;
 }
-constexpr int kCwwMaxE = 511;
-constexpr int kCwcWidths = 5;  // CTA widths 64, 128, 256, 512, 1024
-constexpr int kCwcMbounds = 3;
-__host__ __device__ constexpr int cwc_width(int w) { return 64 << w; }
-__host__ __device__ constexpr int cwc_mbound(int b)
+constexpr int kTeamClasses = 14;
+__host__ __device__ constexpr int team_width_of(int c)
+{
+    return c < 4 ? 0 : c < 8 ? 1 : 2;
+}
+__host__ __device__ constexpr int team_mbound(int c)
+{
+    return c == 0 ? 1024 : c == 1 ? 2048 : c == 2 ? 4096 : c == 3 ? 16384
+         : c == 4 ? 2048 : c == 5 ? 4096 : c == 6 ? 8192 : c == 7 ? 16384
+         : c == 8 ? 4096 : c == 9 ? 6144 : c == 10 ? 8192 : c == 11 ? 10240
+         : c == 12 ? 12288 : 16384;
+}
+constexpr int kTeamMaxE = team_max_e(kTeamWidths - 1);
+constexpr int kTeamMaxM = team_mbound(kTeamClasses - 1);
+constexpr int kIndexClasses = 4;
+__host__ __device__ constexpr int index_max_e(int c)
+{
+    return c == 0 ? 256 : c == 1 ? 1664 : c == 2 ? 4992 : 10016;
+}
+constexpr int kCtaClasses = 3;
+constexpr int kCtaThreads = 1024;
+__host__ __device__ constexpr int cta_mbound(int b)
 {
     return b == 0 ? 16384 : b == 1 ? 65536 : 131072;
 }
-constexpr int kMaxLen = 131072;  // longest pair the CW kernels stage
-constexpr int kClasses = kRwClasses + kCwwClasses + kCwcWidths * kCwcMbounds;
+constexpr int kMaxLen = 131072;  // longest pair routed for E' > 31
+constexpr int kFirstTeam = kRwClasses;
+constexpr int kFirstIndex = kFirstTeam + kTeamClasses;
+constexpr int kFirstCta = kFirstIndex + kIndexClasses;
+constexpr int kClasses = kFirstCta + kCtaClasses;
 constexpr int kLenBins = 72;
 constexpr int kKeys = kClasses * kLenBins;
 
@@ -49,15 +72,28 @@ constexpr int kClassNone = -1;         // m == 0: answered directly
 constexpr int kClassInvalid = -2;      // negative m or E
 constexpr int kClassUnsupported = -3;  // too long for the staged kernels
 
-__host__ __device__ inline int cwc_class(int w, int b)
-{
-    return kRwClasses + kCwwClasses + w * kCwcMbounds + b;
-}
-
 // Effective threshold: rows beyond |s| = m-1 cannot match.
 __host__ __device__ inline int eff_threshold(int m, int E)
 {
     return E < m - 1 ? E : (m > 0 ? m - 1 : 0);
+}
+
+// The class of a pair for the teams or the index (E' up to its largest).
+__host__ __device__ inline int wide_class_of(int m, int Ee)
+{
+    if (Ee <= kTeamMaxE && m <= kTeamMaxM) {
+        int w = 0;
+        while (Ee > team_max_e(w))
+            ++w;
+        int c = 0;
+        while (team_width_of(c) != w || m > team_mbound(c))
+            ++c;
+        return kFirstTeam + c;
+    }
+    int c = 0;
+    while (Ee > index_max_e(c))
+        ++c;
+    return kFirstIndex + c;
 }
 
 __host__ __device__ inline int class_of(int m, int E)
@@ -72,28 +108,22 @@ __host__ __device__ inline int class_of(int m, int E)
             if (Ee <= rw_emax(c))
                 return c;
     }
-    if (Ee <= kCwwMaxE && m <= cww_mbound(kCwwClasses - 1)) {
-        for (int c = 0; c < kCwwClasses; ++c)
-            if (m <= cww_mbound(c))
-                return kRwClasses + c;
-    }
     if (m > kMaxLen)
         return kClassUnsupported;
-    const int words = (2 * Ee + 1 + 31) / 32;
-    int w = 0;
-    while (w < kCwcWidths - 1 && cwc_width(w) < words)
-        ++w;
+    if (Ee <= index_max_e(kIndexClasses - 1))
+        return wide_class_of(m, Ee);
     int b = 0;
-    while (m > cwc_mbound(b))
+    while (m > cta_mbound(b))
         ++b;
-    return cwc_class(w, b);
+    return kFirstCta + b;
 }
 
 // Knobs the autotuner picks (they change speed, never results):
 //   rw_max_e   -- largest E' routed thread-per-pair (15 or 31); above it a
-//                 pair goes to a warp (pairs per warp: 32 -> 1)
-//   cw_subgrid -- columns evaluated bit-parallel across rows before the
-//                 surviving runs are extended word-wise (4, 8 or 16)
+//                 pair goes to a team (pairs per warp: 32 -> 4)
+//   cw_subgrid -- columns the CTA-per-pair kernel evaluates bit-parallel
+//                 across rows before the surviving runs are extended
+//                 word-wise (4, 8 or 16)
 struct TuneParams {
     int rw_max_e = 31;
     int cw_subgrid = 8;
@@ -103,20 +133,9 @@ __host__ __device__ inline int class_of_tuned(int m, int E,
                                               const TuneParams &tp)
 {
     const int c = class_of(m, E);
-    if (c >= 0 && c < kRwClasses && eff_threshold(m, E) > tp.rw_max_e) {
-        // above the thread-per-pair limit: the warp or CTA kernel
-        const int Ee = eff_threshold(m, E);
-        (void)Ee;
-        if (m <= cww_mbound(kCwwClasses - 1)) {
-            for (int k = 0; k < kCwwClasses; ++k)
-                if (m <= cww_mbound(k))
-                    return kRwClasses + k;
-        }
-        int b = 0;
-        while (m > cwc_mbound(b))
-            ++b;
-        return cwc_class(0, b);
-    }
+    // above the thread-per-pair limit: a team, or for long reads the index
+    if (c >= 0 && c < kRwClasses && eff_threshold(m, E) > tp.rw_max_e)
+        return wide_class_of(m, eff_threshold(m, E));
     return c;
 }
 
@@ -202,24 +221,17 @@ struct LongQueue {
 
 constexpr int kLongRing = 1 << 18;   // entries (a power of two)
 constexpr int kLongBatches = 64;     // descriptors
-// Worker shape: one CTA of 512 threads per SM, split into two teams of
-// 256 that each route their own pair, with 72 KB of shared memory each (the
-// longest pair of the served workload, 100 kbp at E = 10^4, needs 70 KB).
-// A/B on GB300, served workload at 2 slots (burst capacity): one pair per
-// CTA of 256 threads 222k pairs/s, of 512 threads 260k; two teams with 48,
-// 64, 72 and 80 KB each 342k, 25k, 374k and 376k -- with 48 KB the longest
-// pairs stayed in their batches' passes, and with 64 KB those passes'
-// kernels no longer fitted beside the worker and waited for it to leave;
-// four teams of 128 threads with 24 KB each 222k.  768 or 1024 threads, or
-// two CTAs per SM, left too little of the SM for the batches' own kernels.
-constexpr int kLongThreads = 512;      // worker CTA width
-constexpr int kLongCtasPerSm = 1;      // worker CTAs per SM
-constexpr int kLongTeams = 2;          // pairs a worker CTA routes at once
-constexpr int kLongWords = 36 * 1024;  // worker shared words per CTA
+// Worker shape: one CTA per SM, routing a pair at a time with an index of up
+// to 98 KB (a pair of 100 kbp at E = 10^4), so that more than half of the
+// SM's shared memory stays free for the batches' own kernels (without room
+// beside the worker they waited for it to leave).
+constexpr int kLongCtasPerSm = 1;
 
-// Whether the queue takes a pair of class cls (m, E'): the CTA-per-pair
-// classes whose staged planes fit the worker's shared memory.
-__host__ __device__ inline bool long_queued(int cls, int m, int Ee);
+// Whether the queue takes the pairs of class cls: the index classes.
+__host__ __device__ inline bool long_queued(int cls)
+{
+    return cls >= kFirstIndex && cls < kFirstCta;
+}
 
 // A batch's hook into the queue: its descriptor index, passed to the
 // enqueue kernel of its pass.

@@ -1,6 +1,6 @@
-// ss_cw.cuh -- K4 for large thresholds: one warp or one CTA per pair, maze
-// bit-parallel across the rows ("column-wise"), with a row-wise extension
-// of the surviving runs.
+// ss_cw.cuh -- K4 for the largest thresholds (E' > 10016): one CTA per
+// pair, maze bit-parallel across the rows ("column-wise"), with a row-wise
+// extension of the surviving runs.
 //
 // Method (Section 2.4): from checkpoint c the greedy needs
 //     p* = max over the 2E+1 rows s of (first obstacle of row s at or after c)
@@ -148,38 +148,21 @@ struct CwArgs {
     int queued = 0;   // skip the pairs the serving queue takes
 };
 
-__host__ __device__ inline bool long_queued(int cls, int m, int Ee)
-{
-    return cls >= kRwClasses + kCwwClasses &&
-           CwLayout::of(m, Ee).words() <= kLongWords / kLongTeams;
-}
-
-// Barrier of a team of nt threads (whole warps) with its own named
-// barrier bar (1..15); bar 0: the whole CTA.
-__device__ __forceinline__ void team_sync(int bar, int nt)
-{
-    if (bar == 0)
-        __syncthreads();
-    else
-        asm volatile("bar.sync %0, %1;" : : "r"(bar), "r"(nt) : "memory");
-}
-
-// Route one pair with a team of nt threads (t: the thread's index in the
-// team; any number of row words): the pair staged into smem, then the
-// greedy of Section 2.4 with one team maximum per step (red: two 32-entry
-// buffers, buf toggles between steps).  Returns min(count, E+1) (count
-// itself is capped by the loop).
+// Route one pair with the whole CTA (any number of row words): the pair
+// staged into smem, then the greedy of Section 2.4 with one CTA maximum per
+// step (red: two 32-entry buffers, buf toggles between steps).  Returns
+// min(count, E+1) (count itself is capped by the loop).
 template <int K>
-__device__ __forceinline__ int cw_team_route(uint32_t *smem, int (*red)[32],
-                                             int &buf, const uint32_t *gq,
-                                             const uint32_t *gr, int m, int E,
-                                             int t, int nt, int bar)
+__device__ __forceinline__ int cw_cta_route(uint32_t *smem, int (*red)[32],
+                                            int &buf, const uint32_t *gq,
+                                            const uint32_t *gr, int m, int E)
 {
+    const int t = threadIdx.x, nt = blockDim.x;
     const int lane = t & 31, warp = t >> 5, nwarp = nt >> 5;
     const int Ee = eff_threshold(m, E);
     const CwLayout L = CwLayout::of(m, Ee);
     cw_stage(smem, L, gq, gr, m, t, nt);
-    team_sync(bar, nt);
+    __syncthreads();
     const int nwords = (2 * Ee + 1 + 31) >> 5;
     int c = 0, count = 0;
     for (;;) {
@@ -189,7 +172,7 @@ __device__ __forceinline__ int cw_team_route(uint32_t *smem, int (*red)[32],
         cand = __reduce_max_sync(0xffffffffu, cand);
         if (lane == 0)
             red[buf][warp] = cand;
-        team_sync(bar, nt);
+        __syncthreads();
         int v = lane < nwarp ? red[buf][lane] : -1;
         const int pstar = __reduce_max_sync(0xffffffffu, v);
         buf ^= 1;
@@ -201,61 +184,6 @@ __device__ __forceinline__ int cw_team_route(uint32_t *smem, int (*red)[32],
         c = pstar + 1;
     }
     return count;
-}
-
-// The same with the whole CTA as the team.
-template <int K>
-__device__ __forceinline__ int cw_cta_route(uint32_t *smem, int (*red)[32],
-                                            int &buf, const uint32_t *gq,
-                                            const uint32_t *gr, int m, int E)
-{
-    return cw_team_route<K>(smem, red, buf, gq, gr, m, E, threadIdx.x,
-                            blockDim.x, 0);
-}
-
-// Warp per pair; blockDim.x / 32 warps, each with its own slice.
-template <int K>
-__global__ void __launch_bounds__(128) k_cw_warp(const CwArgs a)
-{
-    extern __shared__ uint32_t smem[];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    uint32_t *sm = smem + (size_t)warp * a.slice_words;
-    const int begin = a.ws.ranges[2 * a.cls];
-    const int end = a.ws.ranges[2 * a.cls + 1];
-    for (;;) {
-        int idx = 0;
-        if (lane == 0)
-            idx = begin + (int)atomicAdd(&a.ws.counters[a.cls], 1u);
-        idx = __shfl_sync(0xffffffffu, idx, 0);
-        if (idx >= end)
-            break;
-        const int64_t p = a.ws.perm[idx];
-        const int m = a.ps.len(p), E = a.ps.thr(p);
-        const int Ee = eff_threshold(m, E);
-        const CwLayout L = CwLayout::of(m, Ee);
-        const int64_t off = a.ps.off(p);
-        cw_stage(sm, L, a.ps.reads + off, a.ps.refs + off, m, lane, 32);
-        __syncwarp();
-        const int nwords = (2 * Ee + 1 + 31) >> 5;  // <= 32
-        int c = 0, count = 0;
-        for (;;) {
-            const int cand = lane < nwords ? cw_word<K>(sm, L, m, Ee, c, lane)
-                                           : -1;
-            const int pstar = __reduce_max_sync(0xffffffffu, cand);
-            if (pstar >= m)
-                break;  // the net reached the destination
-            ++count;
-            if (count > E)
-                break;
-            c = pstar + 1;
-        }
-        if (lane == 0) {
-            a.ps.acc[p] = (uint8_t)(count <= E);
-            a.ps.obs[p] = count;
-        }
-        __syncwarp();
-    }
 }
 
 // CTA per pair (blockDim.x threads, any number of row words).
@@ -278,10 +206,6 @@ __global__ void __launch_bounds__(1024) k_cw_cta(const CwArgs a)
             break;
         const int64_t p = a.ws.perm[idx];
         const int m = a.ps.len(p), E = a.ps.thr(p);
-        if (a.queued && long_queued(a.cls, m, eff_threshold(m, E))) {
-            __syncthreads();  // s_idx is reused
-            continue;         // routed by the serving queue's worker
-        }
         const int64_t off = a.ps.off(p);
         const int count = cw_cta_route<K>(smem, red, buf, a.ps.reads + off,
                                           a.ps.refs + off, m, E);

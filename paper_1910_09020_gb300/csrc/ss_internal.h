@@ -80,7 +80,6 @@ cudaError_t rw_init(int device);
 // K2 + K4: bucketed persistent form of a mixed batch.
 size_t bucket_ws_bytes(int64_t n);
 BucketWs bucket_ws_at(void *base, int64_t n);
-int cw_class_slice_words(int cls);
 cudaError_t launch_bucketed_one_stream(const PairSet &ps, const BucketWs &ws,
                                        int *status, cudaStream_t st);
 // Kernel attributes and persistent grid sizes of the current device, once

@@ -10,10 +10,10 @@
 // of the SMs, so that a batch admitted while others run executes beside
 // them instead of queueing behind them.
 //
-// Long pairs do not hold a slot.  The pairs of the CTA-per-pair classes
-// (thresholds above 511, or reads past 16 kbp) that fit the worker's shared
-// memory go into a device-resident ring instead of their batch's class
-// kernels, and one long-lived persistent worker kernel (one CTA per SM)
+// Long pairs do not hold a slot.  The pairs of the index classes
+// (thresholds from 497 to 10016, or reads past 16 kbp) go into a
+// device-resident ring instead of their batch's class kernels, and one
+// long-lived persistent worker kernel (one CTA per SM)
 // drains that ring for every batch: a slot frees as soon as its pass ends,
 // while its long pairs run beside later batches' work.  The worker exits
 // after a bounded idle time (or when the server stops) and the scheduler
@@ -40,6 +40,7 @@
 #include "../../include/ss.h"
 #include "ss_bucket.cuh"
 #include "ss_cw.cuh"
+#include "ss_cwx.cuh"
 #include "ss_device.cuh"
 #include "ss_internal.h"
 
@@ -232,44 +233,39 @@ __device__ int long_claim(const ssk::LongQueue &q, uint64_t idle_ns,
     return -1;
 }
 
-// The long-lived worker: each CTA is two teams of 256 threads, and each
-// team takes queued pairs one at a time and routes each (Section 2.4, rows
-// across the team's threads) in its half of the shared memory;
-// the team that routes a batch's last queued pair publishes the batch's
-// generation to the host.  Pairs flagged as holding a non-base get
-// obstacles -1 (their batch's request fails alone, as in the pass).
-__global__ void __launch_bounds__(ssk::kLongThreads)
+// The long-lived worker: each CTA takes queued pairs one at a time and
+// routes each (Section 2.4, by the index of ss_cwx.cuh); the CTA that routes
+// a batch's last queued pair publishes the batch's generation to the host.
+// Pairs flagged as holding a non-base get obstacles -1 (their batch's
+// request fails alone, as in the pass).
+__global__ void __launch_bounds__(ssk::kIndexThreads)
     k_long_worker(const ssk::LongQueue q, uint64_t idle_ns)
 {
-    constexpr int TT = ssk::kLongThreads / ssk::kLongTeams;
     extern __shared__ uint32_t smem[];
-    __shared__ int red[ssk::kLongTeams][2][32];
-    __shared__ int64_t s_pair[ssk::kLongTeams];
-    __shared__ int s_batch[ssk::kLongTeams];
-    const int team = threadIdx.x / TT, t = threadIdx.x % TT;
-    const int bar = 1 + team;  // named barrier of the team
-    uint32_t *slice = smem + team * (ssk::kLongWords / ssk::kLongTeams);
-    int buf = 0;
+    __shared__ ssk::IndexShared s;
+    __shared__ int64_t s_pair;
+    __shared__ int s_batch;
+    const int t = threadIdx.x;
     for (;;) {
         if (t == 0) {
             int64_t p = 0;
-            s_batch[team] = long_claim(q, idle_ns, p);
-            s_pair[team] = p;
+            s_batch = long_claim(q, idle_ns, p);
+            s_pair = p;
         }
-        ssk::team_sync(bar, TT);
-        const int b = s_batch[team];
+        __syncthreads();
+        const int b = s_batch;
         if (b < 0)
             break;
-        const int64_t p = s_pair[team];
+        const int64_t p = s_pair;
         const ssk::PairSet ps = q.batches[b].ps;
         const uint8_t *bad = q.batches[b].bad;
         const int m = ps.len(p), E = ps.thr(p);
         int count = -1;
         if (!(bad && bad[p])) {
             const int64_t off = ps.off(p);
-            count = ssk::cw_team_route<8>(slice, red[team], buf,
-                                          ps.reads + off, ps.refs + off, m, E,
-                                          t, TT, bar);
+            count = ssk::index_route_any(
+                ssk::class_of(m, E) - ssk::kFirstIndex, smem, s,
+                ps.reads + off, ps.refs + off, m, E);
         }
         if (t == 0) {
             ps.acc[p] = (uint8_t)(count >= 0 && count <= E);
@@ -282,11 +278,11 @@ __global__ void __launch_bounds__(ssk::kLongThreads)
             }
             atomicSub(q.busy, 1);
         }
-        ssk::team_sync(bar, TT);  // the slice and s_batch are reused
+        __syncthreads();  // s_batch and the tables are reused
     }
 }
 
-size_t worker_smem() { return (size_t)ssk::kLongWords * 4; }
+size_t worker_smem() { return (size_t)ssk::IndexShape3::WORDS * 4; }
 
 // Launch the worker if work is in flight (want, or queued pairs remain)
 // and none is running.  It is launched ahead of each batch's kernels: its
@@ -299,7 +295,7 @@ void ensure_worker(ss_server *s, bool want = false)
     if (s->worker_launched && cudaEventQuery(s->wev) == cudaErrorNotReady)
         return;
     (void)cudaGetLastError();
-    k_long_worker<<<s->sm_count * ssk::kLongCtasPerSm, ssk::kLongThreads,
+    k_long_worker<<<s->sm_count * ssk::kLongCtasPerSm, ssk::kIndexThreads,
                     worker_smem(), s->wst>>>(s->lq, kWorkerIdleNs);
     if (cudaGetLastError() != cudaSuccess ||
         cudaEventRecord(s->wev, s->wst) != cudaSuccess) {
@@ -462,7 +458,7 @@ int launch_batch(ss_server *s, int slot_idx, std::vector<Request *> &take)
             if (cls < 0)
                 continue;
             counts[cls] += 1;
-            if (ssk::long_queued(cls, m, ssk::eff_threshold(m, E))) {
+            if (ssk::long_queued(cls)) {
                 queued[cls] += 1;
                 ++nlong;
             }
