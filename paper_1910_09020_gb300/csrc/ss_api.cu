@@ -1269,7 +1269,7 @@ int ss_edit_distance_varlen(ss_ctx *ctx, const void *reads, const void *refs,
     DeviceGuard g(ctx->device);
     SS_CUDA(ssk::launch_ed_var((const uint32_t *)reads,
                                (const uint32_t *)refs, offsets, lengths, E,
-                               n, out_ed, ctx->d_status, ctx->sm_count,
+                               n, out_ed, ctx->d_status,
                                pick_stream(stream)));
     ctx->counters.launches += 2;
     return SS_OK;
@@ -1329,6 +1329,14 @@ int ss_filter_submaze(ss_ctx *ctx, const void *reads, const void *refs,
                                            (const uint32_t *)refs, n, m, e,
                                            t, y, out_accept, out_obstacles,
                                            st));
+        ctx->counters.launches += 1;
+        return SS_OK;
+    }
+    if (ssk::pm_submaze_faster(m, e)) {
+        SS_CUDA(ssk::launch_pm_submaze((const uint32_t *)reads,
+                                       (const uint32_t *)refs, n, m, e, t, y,
+                                       out_accept, out_obstacles,
+                                       ctx->sm_count, st));
         ctx->counters.launches += 1;
         return SS_OK;
     }

@@ -320,7 +320,9 @@ cudaError_t bucket_init()
     LaunchCfg &cfg = g_cfg[d];
     if (cfg.ready.load(std::memory_order_relaxed))
         return cudaSuccess;
-    if ((e = rw_init(d)) != cudaSuccess)
+    if ((e = rw_init(d)) != cudaSuccess ||
+        (e = pm_submaze_init()) != cudaSuccess ||
+        (e = pm_ed_init()) != cudaSuccess)
         return e;
     cfg.per_sm[0] = occupancy_per_sm(k_rw_bucket<1>, 128, 0);
     cfg.per_sm[1] = occupancy_per_sm(k_rw_bucket<3>, 128, 0);

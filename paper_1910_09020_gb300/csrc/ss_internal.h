@@ -108,7 +108,21 @@ struct SegArgs;
 size_t seg_smem_bytes();
 cudaError_t launch_seg_direct(const SegArgs &a, cudaStream_t st);
 
-// Accuracy harness (ss_verify.cu): banded edit distance, E <= kEdMaxE.
+// The sub-maze mode over pair-major packed pairs walked bit-sliced
+// (ss_pm_sub.cu), 0 <= E <= kSlicedMaxE, m up to what a CTA stages (else
+// cudaErrorInvalidValue, nothing launched); where it is faster than a thread
+// per pair (m a length it takes).
+cudaError_t launch_pm_submaze(const uint32_t *reads, const uint32_t *refs,
+                              int64_t n, int32_t m, int32_t E, int32_t t,
+                              int32_t y, uint8_t *acc, int32_t *obs,
+                              int sm_count, cudaStream_t st);
+bool pm_submaze_faster(int32_t m, int32_t E);
+// Kernel attributes of that launch and of the bit-sliced distances, on the
+// current device (called by bucket_init under its lock).
+cudaError_t pm_submaze_init();
+cudaError_t pm_ed_init();
+
+// Accuracy harness (ss_verify.cu): capped edit distance, E <= kEdMaxE.
 constexpr int kEdMaxE = 31;
 cudaError_t launch_ed_banded(int E, const uint32_t *reads,
                              const uint32_t *refs, int64_t n, int32_t m,
@@ -118,7 +132,7 @@ constexpr int kEdWarpMaxE = 511;
 cudaError_t launch_ed_var(const uint32_t *reads, const uint32_t *refs,
                           const int64_t *off, const int32_t *len,
                           const int32_t *E, int64_t n, int32_t *ed,
-                          int *status, int sm_count, cudaStream_t st);
+                          int *status, cudaStream_t st);
 cudaError_t launch_confusion(const uint8_t *acc, const int32_t *ed,
                              int64_t n, int E, unsigned long long *counts,
                              int sm_count, cudaStream_t st);

@@ -1,4 +1,4 @@
-// ss_verify.cu -- accuracy harness kernels: banded edit distance per pair
+// ss_verify.cu -- accuracy harness kernels: capped edit distance per pair
 // and the confusion counts of filter decisions against it.
 #include <cuda_runtime.h>
 
@@ -6,18 +6,40 @@
 #include <cstdint>
 
 #include "ss_internal.h"
+#include "ss_pm.cuh"
 #include "ss_verify.cuh"
 
 namespace ssk {
 
+// Pairs of one length and threshold, 32 per thread (ed_walk): 3M pairs of
+// 100 bp at E = 5: 0.111 ms, where a thread per pair evaluating 2E+1 cells a
+// row, ten loads each, took 3.756 ms.
 template <int E>
-__global__ void __launch_bounds__(128) k_ed_banded(const EdArgs a)
+__global__ void __launch_bounds__(kPmThreads) k_pm_ed(const PmArgs a, int32_t *ed,
+                                              int vec)
 {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.n;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t *q = a.reads + p * a.w16;
-        const uint32_t *r = a.refs + p * a.w16;
-        a.ed[p] = ed_banded<E>(q, r, a.m, a.w16);
+    extern __shared__ uint32_t x[];
+    PmSrc src;
+    int64_t p0;
+    int np;
+    if (!pm_prepare(x, a, src, p0, np))
+        return;
+    const uint32_t pad = np >= 32 ? 0u : 0xffffffffu << np;
+    SlicedCount<E> cnt;
+    ed_walk<E>(src, a.m, pad, cnt);
+    uint32_t cb[SlicedShape<E>::NB];
+    cnt.bits(cb);
+    if (np == 32 && vec) {
+        uint4 *o = reinterpret_cast<uint4 *>(ed + p0);
+#pragma unroll
+        for (int v = 0; v < 8; ++v)
+            o[v] = make_uint4((uint32_t)sliced_count<E>(cb, 4 * v),
+                              (uint32_t)sliced_count<E>(cb, 4 * v + 1),
+                              (uint32_t)sliced_count<E>(cb, 4 * v + 2),
+                              (uint32_t)sliced_count<E>(cb, 4 * v + 3));
+    } else {
+        for (int i = 0; i < np; ++i)
+            ed[p0 + i] = sliced_count<E>(cb, i);
     }
 }
 
@@ -57,16 +79,19 @@ __global__ void k_confusion(const uint8_t *__restrict__ acc,
 struct EdVarArgs {
     const uint32_t *reads;
     const uint32_t *refs;
-    const int64_t *off;   // words
-    const int32_t *len;   // bases
-    const int32_t *E;
+    const int64_t *off;   // words; NULL: pair p at word p * ceil(m/16), and
+    const int32_t *len;   // bases;       every pair of m bases
+    const int32_t *E;     //              at threshold e
+    int32_t m, e;
     int64_t n;
     int32_t *ed;
     int *status;
 };
 
 constexpr int kEdVarWarps = 4;
-constexpr int kEdTeamMaxE = 15;  // up to it 8 lanes per pair, above 32
+// up to it 8 lanes per pair, above 32 (1.2M pairs of 250 bp at E = 16 / 31:
+// 32 lanes 1989 / 2984 us, 8 lanes 994 / 2151)
+constexpr int kEdTeamMaxE = 63;
 
 template <int TEAM, int ELO, int EHI>
 __global__ void __launch_bounds__(32 * kEdVarWarps)
@@ -86,8 +111,8 @@ __global__ void __launch_bounds__(32 * kEdVarWarps)
         int m = 0, E = 0;
         bool act = p < a.n;
         if (act) {
-            m = a.len[p];
-            E = a.E[p];
+            m = a.off ? a.len[p] : a.m;
+            E = a.off ? a.E[p] : a.e;
             if (m < 0 || E < 0 || E > kEdWarpMaxE) {
                 if (ELO < 0 && tl == 0) {
                     a.ed[p] = -1;
@@ -101,9 +126,9 @@ __global__ void __launch_bounds__(32 * kEdVarWarps)
         }
         if (!__any_sync(0xffffffffu, act))
             continue;
-        const int64_t off = act ? a.off[p] : 0;
-        const uint32_t *q = a.reads + off, *r = a.refs + off;
         const int w16 = (m + 15) >> 4;
+        const int64_t off = !act ? 0 : a.off ? a.off[p] : p * w16;
+        const uint32_t *q = a.reads + off, *r = a.refs + off;
         for (int x = tl; x < W; x += TEAM)
             F[0][x] = F[1][x] = kEdNone;
         __syncwarp();
@@ -135,26 +160,72 @@ __global__ void __launch_bounds__(32 * kEdVarWarps)
 }
 
 namespace {
-template <int E>
-cudaError_t launch_ed_one(const EdArgs &a, int sm_count, cudaStream_t st)
+
+cudaError_t launch_diag(const EdVarArgs &a, bool small, bool large,
+                        cudaStream_t st)
 {
-    const int64_t want = (a.n + 127) / 128;
-    const int grid = (int)(want < (int64_t)sm_count * 16 ? want
-                                                         : (int64_t)sm_count * 16);
-    k_ed_banded<E><<<grid, 128, 0, st>>>(a);
+    // one warp's worth of pairs per warp (no cap on the grid: pairs differ
+    // in cost by the square of their threshold, and the block scheduler
+    // hands them out as warps finish)
+    auto grid = [&](int teams) {
+        const int64_t per = (int64_t)kEdVarWarps * teams;
+        return (unsigned)std::min<int64_t>((a.n + per - 1) / per, 0x7fffffff);
+    };
+    if (small)
+        k_ed_diag<8, -1, kEdTeamMaxE>
+            <<<grid(4), 32 * kEdVarWarps, 0, st>>>(a);
+    if (large)
+        k_ed_diag<32, kEdTeamMaxE, kEdWarpMaxE>
+            <<<grid(1), 32 * kEdVarWarps, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 template <int... Es>
-cudaError_t launch_ed_dispatch(int E, const EdArgs &a, int sm_count,
-                               cudaStream_t st,
-                               std::integer_sequence<int, Es...>)
+cudaError_t pm_ed_dispatch(int E, const PmArgs &a, int32_t *ed, unsigned grid,
+                           size_t smem, cudaStream_t st,
+                           std::integer_sequence<int, Es...>)
 {
-    cudaError_t out = cudaErrorInvalidValue;
-    ((E == Es ? (out = launch_ed_one<Es>(a, sm_count, st), 0) : 0), ...);
-    return out;
+    const int vec = ((uintptr_t)ed & 15) == 0;
+    cudaError_t r = cudaErrorInvalidValue;
+    ((E == Es ? (k_pm_ed<Es><<<grid, kPmThreads, smem, st>>>(a, ed, vec),
+                 r = cudaGetLastError(), 0)
+              : 0),
+     ...);
+    return r;
 }
+
+template <int... Es>
+cudaError_t pm_ed_attributes(std::integer_sequence<int, Es...>)
+{
+    cudaError_t r = cudaSuccess;
+    ((r == cudaSuccess
+          ? (r = cudaFuncSetAttribute(
+                 k_pm_ed<Es>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                 kPmSmem),
+             0)
+          : 0),
+     ...);
+    return r;
+}
+
+using EdEs = std::make_integer_sequence<int, kEdMaxE + 1>;
+
 }  // namespace
+
+cudaError_t pm_ed_init() { return pm_ed_attributes(EdEs{}); }
+
+// Bit-sliced or by diagonals, whichever is faster: the walk's time grows
+// with the length (twice: a warp holds fewer groups), the diagonals' with
+// the square of the threshold.  Measured (us, walk / diagonals): 3M pairs of
+// 100 bp E = 0 97 / 638, E = 5 115 / 1002; 0.9M of 350 bp E = 0 173 / 207, E
+// = 15 394 / 723; 0.6M of 500 bp E = 5 465 / 248, E = 31 1164 / 1144.  Few
+// pairs leave the walk with a few lanes per warp: 33,000 of 100 bp E = 5 18
+// / 26, of 250 bp E = 5 36 / 26.
+static bool ed_walk_faster(int64_t n, int32_t m)
+{
+    const int w16 = (m + 15) / 16;
+    return w16 <= 22 && n >= (w16 <= 7 ? 16384 : 65536);
+}
 
 cudaError_t launch_ed_banded(int E, const uint32_t *reads,
                              const uint32_t *refs, int64_t n, int32_t m,
@@ -162,30 +233,27 @@ cudaError_t launch_ed_banded(int E, const uint32_t *reads,
 {
     if (n <= 0)
         return cudaSuccess;
-    EdArgs a{reads, refs, n, m, (m + 15) / 16, ed};
-    return launch_ed_dispatch(E, a, sm_count, st,
-                              std::make_integer_sequence<int, kEdMaxE + 1>{});
+    PmArgs a;
+    unsigned grid;
+    size_t smem;
+    if (ed_walk_faster(n, m) &&
+        pm_config(reads, refs, n, m, sm_count, 0, a, grid, smem))
+        return pm_ed_dispatch(E, a, ed, grid, smem, st, EdEs{});
+    const EdVarArgs v{reads, refs, nullptr, nullptr, nullptr, m, E, n, ed,
+                      nullptr};
+    return launch_diag(v, E <= kEdTeamMaxE, E > kEdTeamMaxE, st);
 }
 
 cudaError_t launch_ed_var(const uint32_t *reads, const uint32_t *refs,
                           const int64_t *off, const int32_t *len,
                           const int32_t *E, int64_t n, int32_t *ed,
-                          int *status, int sm_count, cudaStream_t st)
+                          int *status, cudaStream_t st)
 {
     if (n <= 0)
         return cudaSuccess;
-    const EdVarArgs a{reads, refs, off, len, E, n, ed, status};
-    // one warp's worth of pairs per warp (no cap on the grid: pairs differ
-    // in cost by the square of their threshold, and the block scheduler
-    // hands them out as warps finish)
-    auto grid = [n](int teams) {
-        const int64_t per = (int64_t)kEdVarWarps * teams;
-        return (unsigned)std::min<int64_t>((n + per - 1) / per, 0x7fffffff);
-    };
-    k_ed_diag<8, -1, kEdTeamMaxE><<<grid(4), 32 * kEdVarWarps, 0, st>>>(a);
-    k_ed_diag<32, kEdTeamMaxE, kEdWarpMaxE>
-        <<<grid(1), 32 * kEdVarWarps, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_diag(
+        EdVarArgs{reads, refs, off, len, E, 0, 0, n, ed, status}, true, true,
+        st);
 }
 
 cudaError_t launch_confusion(const uint8_t *acc, const int32_t *ed,

@@ -129,9 +129,9 @@ def test_warp_verifier_rejects_out_of_range(F):
     assert g[1] == -1 and g[0] >= 0 and g[2] >= 0
 
 
-@pytest.mark.parametrize("E", [0, 1, 2, 14, 15, 16, 17, 63, 510, 511])
+@pytest.mark.parametrize("E", [0, 1, 2, 15, 16, 62, 63, 64, 65, 510, 511])
 def test_diagonal_verifier_edges(F, E):
-    """Both team widths (E up to 15 and above) at thresholds either side of
+    """Both team widths (E up to 63 and above) at thresholds either side of
     the switch and at the ends of the range, lengths around a packed word
     and below E, related and unrelated pairs, a number of pairs that leaves
     the last warp's teams partly empty."""
@@ -148,3 +148,28 @@ def test_diagonal_verifier_edges(F, E):
             b = refs[off[p]:off[p + 1]].tobytes()
             want = min(oracle.edit_distance(a, b), E + 1)
             assert got[p] == want, (p, int(L[p]), got[p], want)
+
+
+@pytest.mark.parametrize("m,n", [(1, 16384), (33, 20011), (112, 16400),
+                                 (113, 65537), (350, 65536)])
+def test_bit_sliced_distances_equal_the_diagonals(F, m, n):
+    """The bit-sliced walk (from its smallest batches on, lengths either side
+    of its rules' lines, a last group that is not full) against the diagonals
+    over the same pairs as a mixed batch, every pair."""
+    torch = torch_cuda()
+    reads, refs = synth.pairs_fixed(60 + m, 0, n, m, synth.rate_recipe(0.2))
+    refs[::5] = np.roll(reads[::5], 3, axis=0)
+    q = F.pack(to_dev(reads.reshape(-1)), m=m, n=n)
+    r = F.pack(to_dev(refs.reshape(-1)), m=m, n=n)
+    off = torch.arange(n, device="cuda") * binding.ss_packed_words(m)
+    length = torch.full((n,), m, dtype=torch.int32, device="cuda")
+    for E in (0, 1, 6, 15, 31):
+        got = F.edit_distance(q, r, m=m, e=E, n=n)
+        want = F.edit_distance_varlen(q, r, off, length,
+                                      torch.full_like(length, E))
+        F.sync()
+        assert (got == want).all(), (m, E)
+        p = np.random.default_rng(E).integers(0, n, 20)
+        for i in p:
+            ed = oracle.edit_distance(reads[i].tobytes(), refs[i].tobytes())
+            assert int(got[i]) == min(ed, E + 1), (m, E, i)

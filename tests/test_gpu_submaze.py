@@ -111,3 +111,16 @@ def test_submaze_edges(F):
         F.filter_submaze(one, one, m=100, e=40, t=8, y=3, n=1)
     with pytest.raises(binding.SSError):
         F.filter_submaze(one, one, m=100, e=3, t=0, y=3, n=1)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 700])
+@pytest.mark.parametrize("m,E", [(112, 8), (113, 8), (160, 7), (161, 7),
+                                 (256, 16), (257, 16), (100, 0), (100, 31)])
+def test_submaze_either_side_of_the_form_rule(F, n, m, E):
+    """Lengths and thresholds either side of the lines between 32 pairs per
+    thread and one, batches that leave the last group partly empty."""
+    reads, refs = synth.pairs_fixed(900 + m, 0, n, m, synth.rate_recipe(0.1))
+    for t, y in ((8, 3), (m, E + 1)):
+        acc, obs = run(F, reads, refs, E, t, y)
+        oacc, oobs = oracle_submaze(reads, refs, E, t, y)
+        assert_same(acc, obs, oacc, oobs, f"m={m} E={E} t={t} n={n}")
