@@ -373,6 +373,47 @@ cudaError_t rw_init(int device)
     return cudaSuccess;
 }
 
+namespace {
+cudaError_t launch_rw_range(int E, const RwLaunch &L, cudaStream_t st)
+{
+    if (L.grid == 0)
+        return cudaSuccess;
+    if (E <= 9)
+        return launch_rw_uniform_e0(E, L, st);
+    if (E <= 17)
+        return launch_rw_uniform_e1(E, L, st);
+    if (E <= 24)
+        return launch_rw_uniform_e2(E, L, st);
+    return launch_rw_uniform_e3(E, L, st);
+}
+}  // namespace
+
+cudaError_t launch_rw_ascii(int E, const uint8_t *reads, const uint8_t *refs,
+                            int64_t n, int32_t m, uint8_t *acc, int32_t *obs,
+                            int *status, cudaStream_t st)
+{
+    const int64_t ntiles = (n + kRwThreads - 1) / kRwThreads;
+    if (E < 0 || E > kRwMaxE || m < 1 || m > kRwAsciiMaxM ||
+        ntiles > 0x7fffffff)
+        return cudaErrorInvalidValue;
+    RwLaunch L{};
+    L.ascii = true;
+    RwAsciiArgs &a = L.aa;
+    a.reads = reads;
+    a.refs = refs;
+    a.n = n;
+    a.m = m;
+    a.w16 = (m + 15) / 16;
+    a.w16_magic = div_magic((uint32_t)a.w16);
+    a.neg1 = 0xffffffffu;
+    a.acc = acc;
+    a.obs = obs;
+    a.status = status;
+    L.smem = rw_ascii_smem(m, a.w16);
+    L.grid = (unsigned)ntiles;
+    return launch_rw_range(E, L, st);
+}
+
 cudaError_t launch_rw_uniform(int E, const uint32_t *reads,
                               const uint32_t *refs, int64_t n, int32_t m,
                               uint8_t *acc, int32_t *obs, int *status,
@@ -385,7 +426,8 @@ cudaError_t launch_rw_uniform(int E, const uint32_t *reads,
     const int64_t ntiles = (n + kRwThreads - 1) / kRwThreads;
     if (w16 <= kRwPipeMaxW16) {
         L.pipe = true;
-        if (!rw_pipe_config(reads, refs, n, m, acc, obs, status, L.pa,
+        if (!rw_pipe_config(reads, refs, n, m, acc, obs, status,
+                            E < 2 ? kRwSpreadCopies : kRwSpread, L.pa,
                             L.grid, L.smem))
             return cudaErrorInvalidValue;
     } else {
@@ -405,15 +447,7 @@ cudaError_t launch_rw_uniform(int E, const uint32_t *reads,
             return cudaErrorInvalidValue;
         L.grid = (unsigned)ntiles;
     }
-    if (L.grid == 0)
-        return cudaSuccess;
-    if (E <= 9)
-        return launch_rw_uniform_e0(E, L, st);
-    if (E <= 17)
-        return launch_rw_uniform_e1(E, L, st);
-    if (E <= 24)
-        return launch_rw_uniform_e2(E, L, st);
-    return launch_rw_uniform_e3(E, L, st);
+    return launch_rw_range(E, L, st);
 }
 
 }  // namespace ssk
@@ -1005,6 +1039,15 @@ int ss_filter_batch(ss_ctx *ctx, const void *reads, const void *refs,
     if (chunk < 1)
         return SS_ERR_OOM;
     chunk = std::min(chunk, n);
+    // a small batch: packed and filtered in one launch
+    if (!needs_bucket && m <= ssk::kRwAsciiMaxM &&
+        n <= ssk::kRwAsciiMaxBases / m) {
+        SS_CUDA(ssk::launch_rw_ascii(e, (const uint8_t *)reads,
+                                     (const uint8_t *)refs, n, m, out_accept,
+                                     out_obstacles, ctx->d_status, st));
+        ctx->counters.launches += 1;
+        return SS_OK;
+    }
     const size_t bws =
         needs_bucket ? align_up(ssk::bucket_ws_bytes(chunk), 256) : 0;
     const size_t seq_bytes =

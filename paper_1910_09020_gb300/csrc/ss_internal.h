@@ -71,6 +71,16 @@ cudaError_t launch_rw_uniform(int E, const uint32_t *reads,
                               const uint32_t *refs, int64_t n, int32_t m,
                               uint8_t *acc, int32_t *obs, int *status,
                               cudaStream_t st);
+// ASCII pairs packed and filtered by one launch (1 <= m <= kRwAsciiMaxM).
+// Faster than packing to the bit-sliced layout first (two launches, then the
+// walk) up to about kRwAsciiMaxBases bases a side: 100 bp, E = 5, 10 k / 100 k
+// / 400 k pairs 23.7 / 26.9 / 43.3 us -> 10.4 / 16.5 / 44.7; 250 bp, 100 k /
+// 200 k / 400 k 49.4 / 66.0 / 100.6 -> 32.7 / 65.1 / 112.9.
+constexpr int kRwAsciiMaxM = 256;
+constexpr int64_t kRwAsciiMaxBases = 30 * 1000 * 1000;
+cudaError_t launch_rw_ascii(int E, const uint8_t *reads, const uint8_t *refs,
+                            int64_t n, int32_t m, uint8_t *acc, int32_t *obs,
+                            int *status, cudaStream_t st);
 // Devices the one-time set-up below keeps state for (ids 0..63).
 constexpr int kMaxDevices = 64;
 // Kernel attributes of the plain launches on device `device` (the current

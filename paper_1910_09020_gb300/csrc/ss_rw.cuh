@@ -43,6 +43,7 @@
 #include <type_traits>
 
 #include "ss_device.cuh"
+#include "ss_pack.cuh"
 #include "ss_rw_config.h"
 #include "ss_rwc.cuh"
 
@@ -412,7 +413,18 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-constexpr int kRwGroup = 8;                  // tiles per CTA
+constexpr int kRwGroup = 8;                  // tiles per CTA, at most
+// Fewer while the batch has not `spread` times as many tiles: with eight
+// tiles one after another 10,000 pairs (79 tiles) stood on ten SMs, and a
+// batch of a wave or two of CTAs ended with most SMs idle.  Measured at E >=
+// 2 (routing bounds the kernel; the copy of a tile is short) with spread 800
+// / 1600 / 3200 / 6400: 1M pairs of 100 bp, E = 5 70.4 / 62.1 / 60.0 / 59.7
+// us, 1M of 150 bp, E = 7 98.9 / 86.6 / 84.4 / 82.6, 4M of 150 bp 322 / 323
+// / 322 / 318; 10,000 of 100 bp, E = 5 26.9 (always eight) -> 6.3.  At E = 0
+// and 1 the copies bound it, and more tiles per CTA hide them: 1.5M of 250
+// bp, E = 0 50.7 / 49.6 / 49.5 / 57.1.
+constexpr int kRwSpread = 6400;
+constexpr int kRwSpreadCopies = 800;  // E < 2
 constexpr int kRwPipeMaxW16 = 16;            // m <= 256
 constexpr uint64_t kRwWaitNs = 2000000000ull;  // 2 s per stage wait
 
@@ -445,12 +457,12 @@ struct RwPipeArgs {
 };
 
 // Arguments, grid and dynamic shared memory of a pipelined launch over n
-// pairs of length m (w16 <= kRwPipeMaxW16); false if the grid would exceed
-// 2^31 - 1 CTAs.
+// pairs of length m (w16 <= kRwPipeMaxW16), a CTA's tiles by `spread` (see
+// kRwSpread); false if the grid would exceed 2^31 - 1 CTAs.
 inline bool rw_pipe_config(const uint32_t *reads, const uint32_t *refs,
                            int64_t n, int32_t m, uint8_t *acc, int32_t *obs,
-                           int *status, RwPipeArgs &a, unsigned &grid,
-                           size_t &smem)
+                           int *status, int spread, RwPipeArgs &a,
+                           unsigned &grid, size_t &smem)
 {
     const int w16 = (m + 15) / 16 > 1 ? (m + 15) / 16 : 1;
     a.reads = reads;
@@ -459,7 +471,9 @@ inline bool rw_pipe_config(const uint32_t *reads, const uint32_t *refs,
     a.ntiles = (n + kRwThreads - 1) / kRwThreads;
     a.m = m;
     a.w16 = w16;
-    a.group = kRwGroup;
+    a.group = a.ntiles >= (int64_t)kRwGroup * spread
+                  ? kRwGroup
+                  : a.ntiles > spread ? (int32_t)(a.ntiles / spread) : 1;
     a.bulk = ((((uintptr_t)reads) | ((uintptr_t)refs)) & 15) == 0;
     a.neg1 = 0xffffffffu;
     a.acc = acc;
@@ -579,6 +593,115 @@ __global__ void __launch_bounds__(128) k_rw_uniform(const RwPipeArgs a)
                                     const SmemSeqPad &r) {
         return rw_route_plain<E>(q, r, a.m, a.neg1);
     });
+}
+
+// ---- small ASCII batches ----------------------------------------------------
+//
+// A small batch of ASCII pairs costs its launches and the latency of one
+// pair's route, so it takes one launch instead of three: a CTA packs a tile
+// of kRwThreads pairs into shared memory (the arithmetic of ss_pack.cu: the
+// tile's span of a side as 16-byte chunks, each turned into one word of a
+// code stream, and every packed word cut from two of them) and routes it
+// from there, one thread per pair.  10,000 pairs of 100 bp at E = 5: packs
+// 3.2 + 3.3, filter 11.1 us and the gaps between them, 23.7 in all -> 10.4 us.
+struct RwAsciiArgs {
+    const uint8_t *reads;  // pair p at byte p * m
+    const uint8_t *refs;
+    int64_t n;
+    int32_t m;
+    int32_t w16;
+    uint32_t w16_magic;
+    uint32_t neg1;         // 0xffffffff (see rw_route)
+    uint8_t *acc;
+    int32_t *obs;
+    int *status;
+};
+
+// Words of the code stream of a side of a tile: its span, one chunk more on
+// either side, and one (windows read word k + 1).
+SS_HD int rw_ascii_stream(int m) { return kRwThreads * m / 16 + 3; }
+
+// Dynamic shared memory: the stream, then both sides' packed words.
+SS_HD size_t rw_ascii_smem(int m, int w16)
+{
+    return ((size_t)rw_ascii_stream(m) +
+            2u * kRwThreads * (size_t)w16 + kRwPadWords) * 4u;
+}
+
+// Pack pairs p0 .. p0+np-1 of one side into out (pair u at word u * w16).
+__device__ __forceinline__ void rw_ascii_pack(uint32_t *code, uint32_t *out,
+                                              const uint8_t *ascii,
+                                              const RwAsciiArgs &a,
+                                              int64_t p0, int np,
+                                              uint32_t &err)
+{
+    const int t = threadIdx.x;
+    const int64_t b0 = p0 * a.m, limit = a.n * a.m;
+    const int64_t cb = b0 >> 4;  // first chunk
+    const int nc = (int)(((b0 + (int64_t)np * a.m + 15) >> 4) - cb) + 1;
+    const bool aligned = ((uintptr_t)ascii & 15) == 0;
+#pragma unroll 4
+    for (int c = t; c < nc; c += kRwThreads) {
+        const int64_t at = (cb + c) * 16;
+        uint32_t x[4];
+        if (aligned && at + 16 <= limit) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(ascii + at));
+            x[0] = v.x;
+            x[1] = v.y;
+            x[2] = v.z;
+            x[3] = v.w;
+        } else {
+            // the input's last partial chunk, or an unaligned input: bytes
+            // past the end count as 'A'
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t w = 0;
+                for (int b = 0; b < 4; ++b) {
+                    const int64_t j = at + 4 * q + b;
+                    w |= (j < limit ? (uint32_t)__ldg(ascii + j) : 0x41u)
+                         << (8 * b);
+                }
+                x[q] = w;
+            }
+        }
+        code[c] = pack_chunk(x, err);
+    }
+    __syncthreads();
+    const uint32_t o0 = (uint32_t)(b0 - cb * 16);
+    for (int j = t; j < np * a.w16; j += kRwThreads) {
+        const uint32_t u = fast_div((uint32_t)j, (uint32_t)a.w16, a.w16_magic);
+        const uint32_t w = (uint32_t)j - u * (uint32_t)a.w16;
+        const uint32_t o = o0 + u * (uint32_t)a.m + 16u * w;
+        const uint32_t v =
+            pack_window(code[o >> 4], code[(o >> 4) + 1], o & 15u);
+        const uint32_t keep = mask_below(a.m - 16 * (int)w) & 0xffffu;
+        out[j] = v & (keep * 0x10001u);
+    }
+    __syncthreads();
+}
+
+template <int E>
+__global__ void __launch_bounds__(128) k_rw_ascii(const RwAsciiArgs a)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int t = threadIdx.x;
+    const int64_t p0 = (int64_t)blockIdx.x * kRwThreads;
+    const int np = (int)min((int64_t)kRwThreads, a.n - p0);
+    uint32_t *sQ = smem + rw_ascii_stream(a.m);
+    uint32_t *sR = sQ + kRwThreads * a.w16;
+    uint32_t err = 0;
+    // (the stream is read before the second side overwrites it)
+    rw_ascii_pack(smem, sQ, a.reads, a, p0, np, err);
+    rw_ascii_pack(smem, sR, a.refs, a, p0, np, err);
+    if (t < np) {
+        const int cnt = rw_route_plain<E>(SmemSeqPad{sQ + t * a.w16},
+                                          SmemSeqPad{sR + t * a.w16}, a.m,
+                                          a.neg1);
+        a.acc[p0 + t] = (uint8_t)(cnt <= E);
+        a.obs[p0 + t] = cnt;
+    }
+    if (__any_sync(0xffffffffu, err != 0u) && (t & 31) == 0)
+        atomicOr(a.status, kStatusInvalidBase);
 }
 
 }  // namespace ssk

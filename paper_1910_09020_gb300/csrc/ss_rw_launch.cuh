@@ -8,10 +8,11 @@
 
 namespace ssk {
 
-// One plain launch: the persistent pipelined kernel (pipe) or the staged
-// kernel for long reads.
+// One plain launch: the pipelined kernel (pipe), the staged kernel for long
+// reads, or (ascii) the one that packs its pairs itself.
 struct RwLaunch {
-    bool pipe;
+    bool pipe, ascii;
+    RwAsciiArgs aa;
     RwPipeArgs pa;
     RwUniformArgs sa;
     size_t smem;
@@ -21,7 +22,9 @@ struct RwLaunch {
 template <int E>
 cudaError_t rw_launch_one(const RwLaunch &L, cudaStream_t st)
 {
-    if (L.pipe)
+    if (L.ascii)
+        k_rw_ascii<E><<<L.grid, kRwThreads, L.smem, st>>>(L.aa);
+    else if (L.pipe)
         k_rw_uniform<E><<<L.grid, kRwThreads, L.smem, st>>>(L.pa);
     else
         k_rw_staged<E><<<L.grid, kRwThreads, L.smem, st>>>(L.sa);

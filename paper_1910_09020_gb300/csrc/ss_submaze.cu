@@ -70,8 +70,8 @@ cudaError_t submaze_launch_one(const uint32_t *reads, const uint32_t *refs,
         RwPipeArgs a;
         unsigned grid;
         size_t smem;
-        if (!rw_pipe_config(reads, refs, n, m, acc, obs, status, a, grid,
-                            smem))
+        if (!rw_pipe_config(reads, refs, n, m, acc, obs, status, kRwSpread, a,
+                            grid, smem))
             return cudaErrorInvalidValue;
         k_submaze_pipe<EMAX><<<grid, kRwThreads, smem, st>>>(a, E, t, y);
     } else {
