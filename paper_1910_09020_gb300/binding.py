@@ -302,15 +302,15 @@ def _dptr(t, device: int, what: str, nbytes: int = 0) -> int:
         return 0
     if not getattr(t, "is_cuda", False):
         raise ValueError(f"{what}: expected a CUDA tensor on cuda:{device}")
-    if t.device.index != device:
-        raise ValueError(f"{what}: tensor on cuda:{t.device.index}, "
+    if t.get_device() != device:
+        raise ValueError(f"{what}: tensor on cuda:{t.get_device()}, "
                          f"context on cuda:{device}")
     if not t.is_contiguous():
         raise ValueError(f"{what}: tensor must be contiguous")
-    have = t.numel() * t.element_size()
-    if have < nbytes:
-        raise ValueError(f"{what}: {have} bytes, the call needs {nbytes}")
-    return int(t.data_ptr())
+    if nbytes and t.numel() * t.element_size() < nbytes:
+        raise ValueError(f"{what}: {t.numel() * t.element_size()} bytes, "
+                         f"the call needs {nbytes}")
+    return t.data_ptr()
 
 
 def _hptr(t, what: str, nbytes: int = 0) -> int:
@@ -335,10 +335,15 @@ def _seq_bytes(fmt: int, n: int, m: int) -> int:
 
 
 def _stream_handle(stream) -> int:
+    """The stream's handle (None: torch's current stream, asked for without
+    building a Stream object: a call on a small batch is bound by the host)."""
+    if stream is not None:
+        return int(stream.cuda_stream)
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    if torch.cuda.is_initialized():
+        C = torch._C
+        return C._cuda_getCurrentRawStream(C._cuda_getDevice())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 class Filter:
@@ -417,21 +422,27 @@ class Filter:
         import torch
         if n is None:
             n = lengths.shape[0] if lengths is not None else reads.shape[0]
-        dev = reads.device
-        if out_accept is None:
-            out_accept = torch.empty(n, dtype=torch.uint8, device=dev)
-        if out_obstacles is None:
-            out_obstacles = torch.empty(n, dtype=torch.int32, device=dev)
         d = self.device
         seq = _seq_bytes(fmt, n, m) if offsets is None else 0
-        rc = ss_filter_batch(self.ctx, _dptr(reads, d, "reads", seq),
-                             _dptr(refs, d, "refs", seq), fmt,
+        # the inputs first: the results are allocated beside them, and then
+        # need no check
+        pq = _dptr(reads, d, "reads", seq)
+        pr = _dptr(refs, d, "refs", seq)
+        if out_accept is None:
+            out_accept = reads.new_empty(n, dtype=torch.uint8)
+            pa = out_accept.data_ptr()
+        else:
+            pa = _dptr(out_accept, d, "out_accept", n)
+        if out_obstacles is None:
+            out_obstacles = reads.new_empty(n, dtype=torch.int32)
+            po = out_obstacles.data_ptr()
+        else:
+            po = _dptr(out_obstacles, d, "out_obstacles", 4 * n)
+        rc = ss_filter_batch(self.ctx, pq, pr, fmt,
                              _dptr(offsets, d, "offsets", 8 * n),
                              _dptr(lengths, d, "lengths", 4 * n), m,
                              _dptr(E, d, "E", 4 * n), e, n, flags,
-                             _stream_handle(stream),
-                             _dptr(out_accept, d, "out_accept", n),
-                             _dptr(out_obstacles, d, "out_obstacles", 4 * n))
+                             _stream_handle(stream), pa, po)
         _check(rc, "ss_filter_batch")
         if sync:
             self.sync(stream)
