@@ -214,6 +214,7 @@ struct LongQueue {
     unsigned long long *head;    // positions claimed by consumers
     unsigned long long *last;    // time of the last claim by any worker
     int *busy;                   // worker CTAs routing a pair now
+    int *closing;                // set once: every worker CTA leaves
     LongBatch *batches;          // kLongBatches descriptors
     volatile int *done;          // host-mapped: gen of each finished batch
     volatile int *stop;          // host-mapped: workers leave when set

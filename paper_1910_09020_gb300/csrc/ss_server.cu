@@ -184,25 +184,29 @@ __global__ void k_mark_bad(const uint8_t *__restrict__ bad, int64_t n,
         }
 }
 
-// The worker's idle bound: it leaves after this long without a queued pair
-// (long enough to stay through the gaps between requests under load).
-constexpr uint64_t kWorkerIdleNs = 100000000ull;  // 100 ms
+// The worker's idle bound: it leaves after this long without a queued pair.
+// Until it does, whoever waits for the device waits for it, and it holds a
+// share of every SM; a relaunch costs the next batch about 0.1 ms.
+constexpr uint64_t kWorkerIdleNs = 2000000ull;  // 2 ms
 constexpr uint32_t kWorkerMaxPolls = 1u << 22;
 
 // Claim the next published entry of the ring: its batch (>= 0) and pair,
-// or -1 once no worker CTA is routing a pair and none has claimed one for
-// idle_ns (or after kWorkerMaxPolls polls), or the server asked the workers
-// to stop.  So the CTAs leave together: one that left while others still
-// route long pairs would shrink a kernel that keeps running, and the host
-// relaunches only a finished one.  A successful claim counts the CTA busy
-// (the caller ends that with long_done).
+// or -1 once the workers close (no worker CTA routes a pair and none has
+// claimed one for idle_ns, or kWorkerMaxPolls polls), or the server asked
+// them to stop.  The CTA that finds the idle time over closes for all: every
+// CTA leaves at its next claim, also when pairs have been queued meanwhile.
+// (Left to themselves some CTAs left while others took the new pairs, and
+// the host relaunches only a finished kernel: it went on with the few that
+// stayed.)  The host launches the worker again, with closing cleared, as
+// long as queued pairs remain.  A successful claim counts the CTA busy (the
+// caller ends that).
 __device__ int long_claim(const ssk::LongQueue &q, uint64_t idle_ns,
                           int64_t &pair)
 {
     uint64_t t0 = 0;
     uint32_t sleep_ns = 32;
     for (uint32_t polls = 0; polls < kWorkerMaxPolls; ++polls) {
-        if (*q.stop)
+        if (*q.stop || *(volatile int *)q.closing)
             return -1;
         const unsigned long long h =
             *(volatile unsigned long long *)q.head;
@@ -225,11 +229,12 @@ __device__ int long_claim(const ssk::LongQueue &q, uint64_t idle_ns,
         const uint64_t since = last > t0 ? last : t0;
         if (now > since && now - since > idle_ns &&
             *(volatile int *)q.busy == 0)
-            return -1;
+            break;
         __nanosleep(sleep_ns);
         if (sleep_ns < 4096)
             sleep_ns *= 2;
     }
+    *(volatile int *)q.closing = 1;
     return -1;
 }
 
@@ -295,6 +300,12 @@ void ensure_worker(ss_server *s, bool want = false)
     if (s->worker_launched && cudaEventQuery(s->wev) == cudaErrorNotReady)
         return;
     (void)cudaGetLastError();
+    if (cudaMemsetAsync(s->lq.closing, 0, sizeof(int), s->wst) !=
+        cudaSuccess) {
+        (void)cudaGetLastError();
+        s->sticky_error = SS_ERR_CUDA;
+        return;
+    }
     k_long_worker<<<s->sm_count * ssk::kLongCtasPerSm, ssk::kIndexThreads,
                     worker_smem(), s->wst>>>(s->lq, kWorkerIdleNs);
     if (cudaGetLastError() != cudaSuccess ||
@@ -749,6 +760,7 @@ int ss_server_create(ss_server **out, int device, size_t hbm_budget_bytes,
         s->lq.head = (unsigned long long *)(q + ring_bytes + 8);
         s->lq.last = (unsigned long long *)(q + ring_bytes + 16);
         s->lq.busy = (int *)(q + ring_bytes + 24);
+        s->lq.closing = (int *)(q + ring_bytes + 28);
         s->lq.batches = (ssk::LongBatch *)(q + ring_bytes + 256);
         int *hd = nullptr;
         if (cudaHostGetDevicePointer((void **)&hd, s->lq_host, 0) !=
