@@ -24,7 +24,7 @@
 
 #include "ss_bucket.cuh"
 #include "ss_cw.cuh"
-#include "ss_cwt.cuh"
+#include "ss_cws.cuh"
 #include "ss_cwx.cuh"
 #include "ss_device.cuh"
 #include "ss_internal.h"
@@ -218,20 +218,28 @@ BucketWs bucket_ws_at(void *base, int64_t n)
 // Bytes cleared at the start of every pass (hist and ndeferred).
 static size_t bucket_clear_bytes() { return (size_t)kKeys * 4 + 16; }
 
-// Shared memory of a CTA of each team, index and CTA class: its pairs' (the
-// longest the class takes) staged words or tables.
+using RingShape0 = RingShape<512, 512, 128, 2>;
+using RingShape1 = RingShape<1024, 1024, 256>;
+using RingShape2 = RingShape<2048, 1024, 256>;
+static_assert(RingShape0::max_e() >= ring_max_e(0) &&
+                  RingShape1::max_e() >= ring_max_e(1) &&
+                  RingShape2::max_e() >= ring_max_e(2),
+              "a ring class's thresholds fit its rings");
+
+// Shared memory of a CTA of each ring, index and CTA class: its pairs' rings,
+// tables or (the longest the class takes) staged words.
 size_t cw_class_smem(int cls)
 {
-    if (cls < kFirstIndex) {
-        const int c = cls - kFirstTeam;
-        const int pairs = kTeamWarps * 32 / team_lanes(team_width_of(c));
-        return (size_t)pairs * TeamLayout::of(team_mbound(c)).words() * 4;
+    switch (cls - kFirstRing) {
+    case 0: return ring_smem_words<RingShape0>() * 4;
+    case 1: return ring_smem_words<RingShape1>() * 4;
+    case 2: return ring_smem_words<RingShape2>() * 4;
+    default: break;
     }
     switch (cls - kFirstIndex) {
     case 0: return IndexShape0::WORDS * 4;
     case 1: return IndexShape1::WORDS * 4;
     case 2: return IndexShape2::WORDS * 4;
-    case 3: return IndexShape3::WORDS * 4;
     default: break;
     }
     const int M = cta_mbound(cls - kFirstCta);
@@ -283,23 +291,21 @@ const LaunchCfg *launch_cfg()
 
 using CwKernel = void (*)(CwArgs);
 
-// Kernel and CTA width of a team, index or (subgrid k) CTA class.
+// Kernel and CTA width of a ring, index or (subgrid k) CTA class.
 CwKernel cw_kernel(int cls, int k, unsigned &threads)
 {
-    if (cls < kFirstIndex) {
-        threads = 32 * kTeamWarps;
-        switch (team_width_of(cls - kFirstTeam)) {
-        case 0: return k_cw_team<team_lanes(0)>;
-        case 1: return k_cw_team<team_lanes(1)>;
-        default: return k_cw_team<team_lanes(2)>;
-        }
+    threads = 32 * kRingWarps;
+    switch (cls - kFirstRing) {
+    case 0: return k_cw_ring<RingShape0>;
+    case 1: return k_cw_ring<RingShape1>;
+    case 2: return k_cw_ring<RingShape2>;
+    default: break;
     }
     threads = kIndexThreads;
     switch (cls - kFirstIndex) {
     case 0: return k_cw_index<0>;
     case 1: return k_cw_index<1>;
     case 2: return k_cw_index<2>;
-    case 3: return k_cw_index<3>;
     default: break;
     }
     threads = kCtaThreads;
@@ -330,7 +336,7 @@ cudaError_t bucket_init()
     cfg.per_sm[3] = occupancy_per_sm(k_rw_bucket<15>, 128, 0);
     cfg.per_sm[4] = occupancy_per_sm(k_rw_bucket<31>, 128, 0);
     for (int k : {4, 16, 8})
-        for (int cls = kFirstTeam; cls < kClasses; ++cls) {
+        for (int cls = kFirstRing; cls < kClasses; ++cls) {
             unsigned threads = 0;
             const CwKernel f = cw_kernel(cls, k, threads);
             if ((e = cudaFuncSetAttribute(
@@ -467,16 +473,12 @@ cudaError_t launch_cw_classes(const LaunchCfg &cfg, CwArgs a, int subgrid,
                               cudaStream_t st, const int64_t *counts)
 {
     // the index classes first: the pairs that take longest from start to end
-    for (int i = 0; i < kClasses - kFirstTeam; ++i) {
+    for (int i = 0; i < kClasses - kFirstRing; ++i) {
         a.cls = i < kClasses - kFirstIndex ? kFirstIndex + i
-                                           : kFirstTeam + i -
+                                           : kFirstRing + i -
                                                  (kClasses - kFirstIndex);
         if (counts && counts[a.cls] == 0)
             continue;
-        a.slice_words = a.cls < kFirstIndex
-                            ? TeamLayout::of(team_mbound(a.cls - kFirstTeam))
-                                  .words()
-                            : 0;
         unsigned threads = 0;
         const CwKernel f = cw_kernel(a.cls, subgrid, threads);
         const cudaError_t e =
@@ -578,7 +580,7 @@ cudaError_t launch_bucketed(const PairSet &ps, const BucketWs &ws,
         return e;
     *launches += 3;
     const int sh = sm_count;  // persistent grids span this many SMs
-    CwArgs a{ps, ws, 0, 0};
+    CwArgs a{ps, ws, 0};
     if (hook) {
         // serving: the pairs the queue takes
         k_long_enqueue<<<1, 256, 0, st>>>(ps, ws, *hook, hook_expect, status);
@@ -638,7 +640,7 @@ cudaError_t launch_bucketed_one_stream(const PairSet &ps, const BucketWs &ws,
     if ((e = launch_front(ps, ws, tp, status, sm_count, c, st)) !=
         cudaSuccess)
         return e;
-    CwArgs a{ps, ws, 0, 0};
+    CwArgs a{ps, ws, 0};
     if ((e = launch_rw_classes(*cfg, a, sm_count, c, nullptr, st,
                                nullptr)) != cudaSuccess)
         return e;

@@ -6,8 +6,8 @@
 // no Q base at all, so they are all obstacles and never bound the longest
 // run; the count limit still uses E):
 //   * RW classes: E' <= 31, thread per pair, E' <= EMAX in {1, 3, 7, 15, 31}
-//   * team classes: 32 <= E' <= 496 and m <= 16384, 8, 16 or 32 lanes per
-//     pair (ss_cwt.cuh), by team width and m bound
+//   * ring classes: E' <= 816, a team of 2 or 4 lanes per pair (ss_cws.cuh),
+//     by E'
 //   * index classes: E' <= 10016, CTA per pair (ss_cwx.cuh), by E'
 //   * CTA classes: larger E', CTA per pair (ss_cw.cuh), by m bound
 // Within a class pairs are ordered by length, longest first (quarter-octave
@@ -25,34 +25,15 @@ __host__ __device__ constexpr int rw_emax(int c)
 {
     return c == 0 ? 1 : c == 1 ? 3 : c == 2 ? 7 : c == 3 ? 15 : 31;
 }
-// Team classes.  A team's lanes each take one aligned word of 32 starts, and
-// 2E+1 starts touch at most (2E + 31) / 32 + 1 words (rounded down), so
-// teams of 8, 16 and 32 lanes cover a pair up to E' = 112, 240 and 496.  A class's shared-memory slice is sized for its m bound, so
-// finer bounds put more pairs on an SM.
-constexpr int kTeamWidths = 3;
-__host__ __device__ constexpr int team_lanes(int w) { return 8 << w; }
-__host__ __device__ constexpr int team_max_e(int w)
+constexpr int kRingClasses = 3;
+__host__ __device__ constexpr int ring_max_e(int c)
 {
-    return w == 0 ? 112 : w == 1 ? 240 : 496;
+    return c == 0 ? 112 : c == 1 ? 304 : 816;
 }
-constexpr int kTeamClasses = 14;
-__host__ __device__ constexpr int team_width_of(int c)
-{
-    return c < 4 ? 0 : c < 8 ? 1 : 2;
-}
-__host__ __device__ constexpr int team_mbound(int c)
-{
-    return c == 0 ? 1024 : c == 1 ? 2048 : c == 2 ? 4096 : c == 3 ? 16384
-         : c == 4 ? 2048 : c == 5 ? 4096 : c == 6 ? 8192 : c == 7 ? 16384
-         : c == 8 ? 4096 : c == 9 ? 6144 : c == 10 ? 8192 : c == 11 ? 10240
-         : c == 12 ? 12288 : 16384;
-}
-constexpr int kTeamMaxE = team_max_e(kTeamWidths - 1);
-constexpr int kTeamMaxM = team_mbound(kTeamClasses - 1);
-constexpr int kIndexClasses = 4;
+constexpr int kIndexClasses = 3;
 __host__ __device__ constexpr int index_max_e(int c)
 {
-    return c == 0 ? 256 : c == 1 ? 1664 : c == 2 ? 4992 : 10016;
+    return c == 0 ? 1664 : c == 1 ? 5920 : 10016;
 }
 constexpr int kCtaClasses = 3;
 constexpr int kCtaThreads = 1024;
@@ -61,8 +42,8 @@ __host__ __device__ constexpr int cta_mbound(int b)
     return b == 0 ? 16384 : b == 1 ? 65536 : 131072;
 }
 constexpr int kMaxLen = 131072;  // longest pair routed for E' > 31
-constexpr int kFirstTeam = kRwClasses;
-constexpr int kFirstIndex = kFirstTeam + kTeamClasses;
+constexpr int kFirstRing = kRwClasses;
+constexpr int kFirstIndex = kFirstRing + kRingClasses;
 constexpr int kFirstCta = kFirstIndex + kIndexClasses;
 constexpr int kClasses = kFirstCta + kCtaClasses;
 constexpr int kLenBins = 72;
@@ -78,19 +59,15 @@ __host__ __device__ inline int eff_threshold(int m, int E)
     return E < m - 1 ? E : (m > 0 ? m - 1 : 0);
 }
 
-// The class of a pair for the teams or the index (E' up to its largest).
-__host__ __device__ inline int wide_class_of(int m, int Ee)
+// The class of a pair for the ring teams or the index (E' up to its largest).
+__host__ __device__ inline int wide_class_of(int Ee)
 {
-    if (Ee <= kTeamMaxE && m <= kTeamMaxM) {
-        int w = 0;
-        while (Ee > team_max_e(w))
-            ++w;
-        int c = 0;
-        while (team_width_of(c) != w || m > team_mbound(c))
-            ++c;
-        return kFirstTeam + c;
-    }
     int c = 0;
+    if (Ee <= ring_max_e(kRingClasses - 1)) {
+        while (Ee > ring_max_e(c))
+            ++c;
+        return kFirstRing + c;
+    }
     while (Ee > index_max_e(c))
         ++c;
     return kFirstIndex + c;
@@ -111,7 +88,7 @@ __host__ __device__ inline int class_of(int m, int E)
     if (m > kMaxLen)
         return kClassUnsupported;
     if (Ee <= index_max_e(kIndexClasses - 1))
-        return wide_class_of(m, Ee);
+        return wide_class_of(Ee);
     int b = 0;
     while (m > cta_mbound(b))
         ++b;
@@ -120,7 +97,7 @@ __host__ __device__ inline int class_of(int m, int E)
 
 // Knobs the autotuner picks (they change speed, never results):
 //   rw_max_e   -- largest E' routed thread-per-pair (15 or 31); above it a
-//                 pair goes to a team (pairs per warp: 32 -> 4)
+//                 pair goes to a team (pairs per warp: 32 -> 16)
 //   cw_subgrid -- columns the CTA-per-pair kernel evaluates bit-parallel
 //                 across rows before the surviving runs are extended
 //                 word-wise (4, 8 or 16)
@@ -133,9 +110,9 @@ __host__ __device__ inline int class_of_tuned(int m, int E,
                                               const TuneParams &tp)
 {
     const int c = class_of(m, E);
-    // above the thread-per-pair limit: a team, or for long reads the index
+    // above the thread-per-pair limit: a team
     if (c >= 0 && c < kRwClasses && eff_threshold(m, E) > tp.rw_max_e)
-        return wide_class_of(m, eff_threshold(m, E));
+        return wide_class_of(eff_threshold(m, E));
     return c;
 }
 

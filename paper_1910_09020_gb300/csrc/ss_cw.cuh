@@ -143,7 +143,6 @@ struct CwArgs {
     PairSet ps;
     BucketWs ws;
     int cls;
-    int slice_words;  // shared words per staged pair
     uint32_t neg1 = 0xffffffffu;  // passed at run time (see rw_route)
     int queued = 0;   // skip the pairs the serving queue takes
 };

@@ -1,6 +1,6 @@
-// ss_cwx.cuh -- K4 for larger thresholds (E' to 10016) and for long reads
-// (m > 16384): a CTA per pair, which looks the longest escape segments up
-// in an index of the query instead of evaluating the maze rows.
+// ss_cwx.cuh -- K4 for thresholds from 817 to 10016: a CTA per pair, which
+// looks the longest escape segments up in an index of the query instead of
+// evaluating the maze rows.
 //
 // Method (Section 2.4): from checkpoint c the longest escape segment is the
 // longest match of R[c..] with the query from any start j in c-E..c+E.  At
@@ -41,7 +41,7 @@
 
 #include "ss_bucket.cuh"
 #include "ss_cw.cuh"
-#include "ss_cwt.cuh"
+#include "ss_cws.cuh"
 #include "ss_device.cuh"
 
 namespace ssk {
@@ -65,16 +65,19 @@ struct IndexShape {
     static_assert(K >= 2 && K <= 14, "a K-mer and two bases in 32 bits");
 };
 
-// Code bits of the 17 to 32 bases a sequence's words hold from base j on
-// (the number in n): bit t of lo/hi is base j + t.
-SS_HD void base_window(const uint32_t *g, int w16, int j, uint32_t &lo,
-                       uint32_t &hi, int &n)
+// A packed word (code bit 0 of base t at bit t, code bit 1 at bit 16 + t)
+// with the two bits of each base side by side: base t at bits 2t, 2t + 1
+// (the outer perfect shuffle).
+SS_HD uint32_t interleave_codes(uint32_t x)
 {
-    const int i = j >> 4, s = j & 15;
-    const uint32_t a = ldg(g + i), b = i + 1 < w16 ? ldg(g + i + 1) : 0u;
-    lo = prmt(a, b, 0x5410u) >> s;
-    hi = prmt(a, b, 0x7632u) >> s;
-    n = 32 - s;
+    uint32_t t = (x ^ (x >> 8)) & 0x0000ff00u;
+    x ^= t ^ (t << 8);
+    t = (x ^ (x >> 4)) & 0x00f000f0u;
+    x ^= t ^ (t << 4);
+    t = (x ^ (x >> 2)) & 0x0c0c0c0cu;
+    x ^= t ^ (t << 2);
+    t = (x ^ (x >> 1)) & 0x22222222u;
+    return x ^ t ^ (t << 1);
 }
 
 // 16 bases, two bits each, the first in the two highest bits: from a packed
@@ -111,31 +114,6 @@ template <int K>
 SS_HD uint32_t next_two(uint32_t bases)
 {
     return ((bases << (2 * K)) >> 16) & 0xf000u;
-}
-
-// Matching bases of q[j..] and r[c..], at most lim (inside both), over at
-// most `windows` windows: kRunOpen + the bases compared if all of them
-// match and more are left.  rlo, rhi, rn: the window of r at c.
-constexpr int kRunOpen = 1 << 24;
-SS_HD int index_run(const uint32_t *q, const uint32_t *r, int w16, int j,
-                    int c, int lim, uint32_t rlo, uint32_t rhi, int rn,
-                    int windows)
-{
-    int run = 0;
-    for (;;) {
-        uint32_t lo, hi;
-        int n;
-        base_window(q, w16, j + run, lo, hi, n);
-        n = imin(n, rn);
-        const uint32_t x = (lo ^ rlo) | (hi ^ rhi);
-        const int k = imin(x ? ffs32(x) - 1 : 32, n);
-        run += k;
-        if (k < n || run >= lim)
-            return imin(run, lim);
-        if (--windows == 0)
-            return run + kRunOpen;
-        base_window(r, w16, c + run, rlo, rhi, rn);
-    }
 }
 
 // One more start of K-mer x in a table's counts (two 16-bit counts per
@@ -460,15 +438,13 @@ SS_HD void chain_follow(IndexChain &s, const int *col, int c0, int cols,
 }
 
 // The classes' shapes: one to five starts per K-mer and window.
-using IndexShape0 = IndexShape<4, 9, 3>;   // E' <= 256:   4.5 KB
-using IndexShape1 = IndexShape<5, 11, 3>;  // E' <= 1664:   18 KB
-using IndexShape2 = IndexShape<6, 12, 4>;  // E' <= 4992:   64 KB
-using IndexShape3 = IndexShape<6, 12, 6>;  // E' <= 10016:  96 KB
+using IndexShape0 = IndexShape<5, 11, 3>;  // E' <= 1664:   18 KB
+using IndexShape1 = IndexShape<6, 12, 4>;  // E' <= 5920:   64 KB
+using IndexShape2 = IndexShape<6, 12, 6>;  // E' <= 10016:  96 KB
 
 static_assert(IndexShape0::max_e() >= index_max_e(0) &&
                   IndexShape1::max_e() >= index_max_e(1) &&
-                  IndexShape2::max_e() >= index_max_e(2) &&
-                  IndexShape3::max_e() >= index_max_e(3),
+                  IndexShape2::max_e() >= index_max_e(2),
               "a class's thresholds fit its tables");
 
 template <int C>
@@ -479,8 +455,6 @@ template <>
 struct IndexClass<1> { using Shape = IndexShape1; };
 template <>
 struct IndexClass<2> { using Shape = IndexShape2; };
-template <>
-struct IndexClass<3> { using Shape = IndexShape3; };
 
 #ifdef __CUDACC__
 // What the threads of a CTA share besides the tables.
@@ -580,8 +554,7 @@ __device__ __forceinline__ int index_route_any(int ic, uint32_t *tabs,
     switch (ic) {
     case 0: return index_route<IndexShape0>(tabs, s, q, r, m, E);
     case 1: return index_route<IndexShape1>(tabs, s, q, r, m, E);
-    case 2: return index_route<IndexShape2>(tabs, s, q, r, m, E);
-    default: return index_route<IndexShape3>(tabs, s, q, r, m, E);
+    default: return index_route<IndexShape2>(tabs, s, q, r, m, E);
     }
 }
 

@@ -11,7 +11,7 @@
 // them instead of queueing behind them.
 //
 // Long pairs do not hold a slot.  The pairs of the index classes
-// (thresholds from 497 to 10016, or reads past 16 kbp) go into a
+// (thresholds from 817 to 10016) go into a
 // device-resident ring instead of their batch's class kernels, and one
 // long-lived persistent worker kernel (one CTA per SM)
 // drains that ring for every batch: a slot frees as soon as its pass ends,
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(ssk::kIndexThreads)
     }
 }
 
-size_t worker_smem() { return (size_t)ssk::IndexShape3::WORDS * 4; }
+size_t worker_smem() { return (size_t)ssk::IndexShape2::WORDS * 4; }
 
 // Launch the worker if work is in flight (want, or queued pairs remain)
 // and none is running.  It is launched ahead of each batch's kernels: its

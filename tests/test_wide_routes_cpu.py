@@ -1,4 +1,4 @@
-"""Host builds of the team and index routes (thresholds above 31) against the
+"""Host builds of the ring and index routes (thresholds above 31) against the
 oracle, and the class table that chooses between them."""
 import ctypes
 import os
@@ -37,7 +37,7 @@ def emu():
         os.replace(tmp, out)
     lib = ctypes.CDLL(out)
     P, I = ctypes.c_void_p, ctypes.c_int
-    lib.emu_team.argtypes = [P, P, I, I, I]
+    lib.emu_ring.argtypes = [P, P, I, I, I]
     lib.emu_index.argtypes = [P, P, I, I, I]
     lib.emu_wide_class.argtypes = [I, I, I]
     lib.emu_class_table.argtypes = [I, I]
@@ -70,43 +70,45 @@ def some_pairs(seed, m):
 
 
 @pytest.mark.parametrize("m", [1, 2, 3, 4, 5, 15, 16, 17, 31, 32, 33, 63, 64,
-                               65, 96, 127, 160, 700])
-def test_team_route_matches_oracle(emu, m):
+                               65, 96, 127, 160, 255, 256, 257, 448, 700])
+def test_ring_route_matches_oracle(emu, m):
+    """Lengths around the words, the last four columns and the ring's blocks
+    (128 and 256 bases), small and clamped thresholds, every class."""
     for q, r in some_pairs(10 * m, m):
         qw, rw = packed(q), packed(r)
         for E in sorted({0, 1, 16, 31, 32, m // 10, m // 2, m + 3}):
-            if E > 496:
-                continue
             want = oracle.filter_pair(q, r, E).obstacles
-            for lanes in (8, 32):
-                if (2 * min(E, m - 1) + 31) // 32 + 1 > lanes:
-                    continue
-                got = emu.emu_team(ptr(qw), ptr(rw), m, E, lanes)
-                assert got == want, (m, E, lanes, q, r)
+            for rc in (0, 1, 2):
+                if min(E, m - 1) <= emu.emu_class_table(4, rc):
+                    got = emu.emu_ring(ptr(qw), ptr(rw), m, E, rc)
+                    assert got == want, (m, E, rc, q, r)
 
 
-@pytest.mark.parametrize("E", [111, 112, 113, 239, 240, 241, 495, 496])
-def test_team_route_at_width_bounds(emu, E):
-    m = 1200
-    for q, r in some_pairs(E, m):
-        want = oracle.filter_pair(q, r, E).obstacles
-        lanes = 8 if E <= 112 else 16 if E <= 240 else 32
-        qw, rw = packed(q), packed(r)
-        got = emu.emu_team(ptr(qw), ptr(rw), m, E, lanes)
-        assert got == want, (E, q, r)
+@pytest.mark.parametrize("E", [32, 111, 112, 113, 303, 304, 305, 500, 815,
+                               816])
+def test_ring_route_at_class_bounds(emu, E):
+    """Pairs of many ring blocks at thresholds up to the largest of each
+    class (where the window, what is read past it and a block fill the
+    ring)."""
+    rc = sum(E > emu.emu_class_table(4, k) for k in (0, 1))
+    for m in (1200, 6000):
+        for q, r in some_pairs(E + m, m):
+            qw, rw = packed(q), packed(r)
+            want = oracle.filter_pair(q, r, E).obstacles
+            assert emu.emu_ring(ptr(qw), ptr(rw), m, E, rc) == want, (E, m)
 
 
-@pytest.mark.parametrize("ic", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("ic", [0, 1, 2, 3])
 def test_index_route_matches_oracle(emu, ic):
     """Every index shape, from thresholds far below to the largest its ring
     covers, lengths around the blocks (the small shape's ring of four
     blocks of 16 starts turns every 16 columns)."""
-    top = 16 if ic == 4 else emu.emu_class_table(6, ic)
-    block = (512, 2048, 4096, 4096, 16)[ic]
+    top = 16 if ic == 3 else emu.emu_class_table(5, ic)
+    block = (2048, 4096, 4096, 16)[ic]
     lengths = {1, 2, 5, 16, block - 1, block, block + 1, 3 * block + 7}
-    if ic == 4:
-        lengths |= {100, 700}
     if ic == 3:
+        lengths |= {100, 700}
+    if ic == 2:
         lengths = {1, 7, block - 1, block + 1}
     for m in sorted(lengths):
         for k, (q, r) in enumerate(some_pairs(100 * ic + m, m)):
@@ -122,39 +124,32 @@ def test_index_route_matches_oracle(emu, ic):
 
 
 def test_index_ring_past_its_blocks(emu):
-    """A long pair whose window passes over every slot of the ring several
-    times, at the largest threshold of the class."""
-    m = 6000
-    for ic, E in ((0, 256), (1, 1664)):
-        for q, r in some_pairs(900 + ic, m)[:4]:
-            want = oracle.filter_pair(q, r, E).obstacles
-            qw, rw = packed(q), packed(r)
-            got = emu.emu_index(ptr(qw), ptr(rw), m, E, ic)
-            assert got == want, (ic, E)
+    """A long pair whose window passes over every slot of the ring, at the
+    largest threshold of the class."""
+    m, E = 13000, 1664
+    for q, r in some_pairs(900, m)[:4]:
+        want = oracle.filter_pair(q, r, E).obstacles
+        qw, rw = packed(q), packed(r)
+        assert emu.emu_index(ptr(qw), ptr(rw), m, E, 0) == want
 
 
 def test_class_table(emu):
     """Every (m, E') above 31 lands in a class whose bounds hold it."""
     T = emu.emu_class_table
-    team, index, cta, classes = T(0, 0), T(1, 0), T(2, 0), T(7, 0)
-    for m in (33, 100, 1024, 1025, 2048, 2049, 4096, 4097, 6145, 8192, 10241,
-              12289, 16384, 16385, 65537, 131072):
-        for E in (16, 31, 32, 112, 113, 240, 241, 496, 497, 1664, 1665, 4992,
-                  4993, 10016, 10017, 131071):
+    ring, index, cta, classes = (T(k, 0) for k in range(4))
+    for m in (33, 100, 1024, 1025, 16384, 16385, 65537, 131072):
+        for E in (16, 31, 32, 112, 113, 304, 305, 816, 817, 1664, 1665, 5920,
+                  5921, 10016, 10017, 131071):
             for rmax in (15, 31):
                 e = min(E, m - 1)
                 c = emu.emu_wide_class(m, E, rmax)
                 assert 0 <= c < classes
-                if c < team:
+                if c < ring:
                     assert e <= rmax
                 elif c < index:
-                    k = c - team
-                    assert m <= T(4, k) and rmax < e <= T(5, k)
-                    # one word per lane
-                    assert (2 * e + 31) // 32 + 1 <= T(3, k)
+                    assert rmax < e <= T(4, c - ring)
                 elif c < cta:
-                    assert e <= T(6, c - index)
-                    assert e > 496 or m > 16384
+                    assert T(4, 2) < e <= T(5, c - index)
                 else:
                     assert e > 10016
     assert emu.emu_wide_class(131073, 32, 31) == -3
