@@ -7,18 +7,23 @@
 // Why: a pair costs a thread of its own some ops per cell or column, the
 // walk of 32 pairs per word a 32nd of that, and turning 32 words of 16 bases
 // costs about 210 ops, 6.5 per word and pair: 91 a pair of 100 bp.
-// Staging: lane i copies pair i's words (4-byte asynchronous copies), so that
-// the 16 bases' words of a group's 32 pairs end up side by side; the turn and
-// the walk then read and write one lane's region, whose stride is odd,
-// without bank conflicts, and no lane exchanges anything with another.
+// Staging: 4-byte asynchronous copies, 32 consecutive words of a group at a
+// time, each to its place, so that the 16 bases' words of a group's 32 pairs
+// end up side by side; the turn and the walk then read and write one lane's
+// region, whose stride is odd, without bank conflicts, and no lane exchanges
+// anything with another.  (With lane i copying pair i's words a copy touched
+// about w16 + 1 lines: exact distances of 3M pairs of 100 bp, E = 0 / 5 93 /
+// 112 -> 83 / 102 us, 1.2M of 250 bp 151 / 210 -> 118 / 178, sub-mazes of 3M
+// of 100 bp, E = 5 137 -> 127.)
 // One warp per CTA and up to 56 KB of shared memory, so that four CTAs stand
 // on an SM, one per scheduler: a pair's 2 bits per base set how many can be
 // in flight, so a walk lives from the independence of its rows, and the
-// staging of one CTA overlaps the walks of the others.  Bound by the copies
-// (each touches about w16 + 1 lines) at small E, by the issue of one warp
-// per scheduler at large E.
+// staging of one CTA overlaps the walks of the others.  Bound by the issue
+// of one warp per scheduler: 0.31 to 0.36 instructions a cycle (E = 0 and 5),
+// where the logic pipe takes one every two, and a sixth of the time waits for
+// the staged words.
 // What else was measured, exact distances of 3M pairs of 100 bp at E = 0 /
-// 31 (this form: 92 / 233 us): words copied as they lie in memory and turned
+// 31 (this form, before the copies went by lines: 92 / 233 us): words copied as they lie in memory and turned
 // in their places, every later address a multiple of w16: 140 / 281; two
 // warps per CTA, one side each, then one walking (the walking warps of all
 // CTAs on two schedulers): 93 / 354; words turned in registers, 16 bases at
@@ -70,6 +75,11 @@ SS_HD void transpose32(uint32_t (&a)[32])
 // pair, later one per code bit and base), and one to make the stride odd.
 SS_HD int pm_stride(int w16) { return 32 * w16 + 1; }
 
+// Where a region holds word c of its pair i until the turn: the words of
+// consecutive pairs are copied side by side, and would fall w16 to a bank
+// (32c + i); fours of pairs change places by c, which leaves about two.
+SS_HD int pm_place(int c, int i) { return 32 * c + (i ^ (4 * (c & 7))); }
+
 // Turn a region's w16 chunks into bit-sliced words: word 32c + 16b + t is
 // code bit b of base 16c + t, one pair per bit.
 SS_HD void pm_turn(uint32_t *x, int w16)
@@ -77,8 +87,13 @@ SS_HD void pm_turn(uint32_t *x, int w16)
     for (int c = 0; c < w16; ++c) {
         uint32_t a[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-            a[i] = x[32 * c + i];
+        for (int i = 0; i < 32; i += 4) {
+            const uint32_t *p = x + pm_place(c, i);
+            a[i] = p[0];
+            a[i + 1] = p[1];
+            a[i + 2] = p[2];
+            a[i + 3] = p[3];
+        }
         transpose32(a);
 #pragma unroll
         for (int i = 0; i < 32; ++i)
@@ -256,27 +271,46 @@ struct PmArgs {
 
 constexpr int kPmThreads = 32;
 
-// Stage G groups of one side in x (src: the words of the first one's pairs,
-// pairs of them exist): lane i the pairs 32g + i; words of pairs that do not
-// exist are zero.
-__device__ __forceinline__ void pm_stage(uint32_t *x, const uint32_t *src,
-                                         int64_t pairs, int G, int w16)
+// Stage G groups of both sides, the reads' regions at x, the references'
+// after them (q, r: the words of the first group's pairs, pairs of them
+// exist): a group's words as they follow one another in memory, 32 per copy;
+// words of pairs that do not exist are zero.
+__device__ __forceinline__ void pm_stage(uint32_t *x, const uint32_t *q,
+                                         const uint32_t *r, int64_t pairs,
+                                         int G, int w16)
 {
     const int lane = threadIdx.x, stride = pm_stride(w16);
-    for (int g = 0; g < G; ++g) {
-        uint32_t *to = x + g * stride + lane;
-        if (32 * g + lane < pairs) {
-            const uint32_t at = smem_addr(to);
-            const uint32_t *from = src + (int64_t)(32 * g + lane) * w16;
+    const int full = (int)min((int64_t)G, pairs >> 5);
+    const int du = 32 / w16, dc = 32 % w16;
+    int u = lane / w16, c = lane % w16;  // word 32k + lane: pair, word of it
+    for (int k = 0; k < w16; ++k) {
+        uint32_t *to = x + pm_place(c, u);
+        uint32_t at = smem_addr(to);
+        int from = 32 * k + lane;
 #pragma unroll 4
-            for (int c = 0; c < w16; ++c)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                                 at + 128 * c),
-                             "l"(from + c)
-                             : "memory");
-        } else {
-            for (int c = 0; c < w16; ++c)
-                to[32 * c] = 0u;
+        for (int g = 0; g < full; ++g) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(at),
+                         "l"(q + from)
+                         : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                             at + 4 * G * stride),
+                         "l"(r + from)
+                         : "memory");
+            at += 4 * stride;
+            from += 32 * w16;
+        }
+        // the batch's last pairs, and groups past it
+        for (int g = full; g < G; ++g) {
+            const bool exists = 32 * g + u < pairs;
+            const int at_word = (32 * g + u) * w16 + c;
+            to[g * stride] = exists ? q[at_word] : 0u;
+            to[(G + g) * stride] = exists ? r[at_word] : 0u;
+        }
+        u += du;
+        c += dc;
+        if (c >= w16) {
+            c -= w16;
+            ++u;
         }
     }
 }
@@ -288,8 +322,8 @@ __device__ __forceinline__ bool pm_prepare(uint32_t *x, const PmArgs &a,
 {
     const int lane = threadIdx.x, stride = pm_stride(a.w16);
     const int64_t first = (int64_t)blockIdx.x * a.G * 32;
-    pm_stage(x, a.q + first * a.w16, a.n - first, a.G, a.w16);
-    pm_stage(x + a.G * stride, a.r + first * a.w16, a.n - first, a.G, a.w16);
+    pm_stage(x, a.q + first * a.w16, a.r + first * a.w16, a.n - first, a.G,
+             a.w16);
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::
                      : "memory");
     __syncwarp();

@@ -77,11 +77,12 @@ using AllE = std::make_integer_sequence<int, kSlicedMaxE + 1>;
 
 cudaError_t pm_submaze_init() { return pm_attributes(AllE{}); }
 
-// Against a thread per pair (k_submaze_pipe), t = 8, y = 3, 3M pairs of 100
-// bp (2M of 150, 1.2M of 250): E = 0 102 -> 101 us (109 -> 116), E = 5 244
-// -> 134 (227 -> 166; 265 -> 269), E = 10 269 -> 160 (241 -> 268), E = 20
-// 1314 -> 244 (1077 -> 273; 999 -> 439).  A warp holds fewer groups the
-// longer the pairs, and the thread per pair has no column walk above E = 15.
+// Against a thread per pair (k_submaze_pipe), t = 8, y = 3, in us (thread ->
+// walk), 3M pairs of 100 bp; 2M of 150; 1.2M of 250: E = 0 92 -> 96; 84 ->
+// 113; 98 -> 144, E = 5 244 -> 127; 227 -> 160; 223 -> 232, E = 10 269 ->
+// 151; 239 -> 254; 240 -> 288, E = 20 1314 -> 229; 1077 -> 268; 999 -> 399.
+// A warp holds fewer groups the longer the pairs, and the thread per pair
+// has no column walk above E = 15.
 bool pm_submaze_faster(int32_t m, int32_t E)
 {
     const int w16 = (m + 15) / 16;

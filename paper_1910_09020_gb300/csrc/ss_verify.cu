@@ -12,7 +12,7 @@
 namespace ssk {
 
 // Pairs of one length and threshold, 32 per thread (ed_walk): 3M pairs of
-// 100 bp at E = 5: 0.111 ms, where a thread per pair evaluating 2E+1 cells a
+// 100 bp at E = 5: 0.102 ms, where a thread per pair evaluating 2E+1 cells a
 // row, ten loads each, took 3.756 ms.
 template <int E>
 __global__ void __launch_bounds__(kPmThreads) k_pm_ed(const PmArgs a, int32_t *ed,
@@ -217,8 +217,8 @@ cudaError_t pm_ed_init() { return pm_ed_attributes(EdEs{}); }
 // Bit-sliced or by diagonals, whichever is faster: the walk's time grows
 // with the length (twice: a warp holds fewer groups), the diagonals' with
 // the square of the threshold.  Measured (us, walk / diagonals): 3M pairs of
-// 100 bp E = 0 97 / 638, E = 5 115 / 1002; 0.9M of 350 bp E = 0 173 / 207, E
-// = 15 394 / 723; 0.6M of 500 bp E = 5 465 / 248, E = 31 1164 / 1144.  Few
+// 100 bp E = 0 83 / 638, E = 5 102 / 1002; 0.9M of 350 bp E = 0 141 / 207, E
+// = 15 390 / 723; 0.6M of 500 bp E = 5 465 / 248, E = 31 1164 / 1144.  Few
 // pairs leave the walk with a few lanes per warp: 33,000 of 100 bp E = 5 18
 // / 26, of 250 bp E = 5 36 / 26.
 static bool ed_walk_faster(int64_t n, int32_t m)

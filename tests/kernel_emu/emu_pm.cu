@@ -21,7 +21,7 @@ std::vector<uint32_t> region(const uint32_t *x, int64_t n, int64_t p0,
     std::vector<uint32_t> out(pm_stride(w16), 0u);
     for (int i = 0; i < 32 && p0 + i < n; ++i)
         for (int c = 0; c < w16; ++c)
-            out[32 * c + i] = x[(p0 + i) * w16 + c];
+            out[pm_place(c, i)] = x[(p0 + i) * w16 + c];
     pm_turn(out.data(), w16);
     return out;
 }
