@@ -59,11 +59,13 @@ __host__ __device__ inline int eff_threshold(int m, int E)
     return E < m - 1 ? E : (m > 0 ? m - 1 : 0);
 }
 
-// The class of a pair for the ring teams or the index (E' up to its largest).
-__host__ __device__ inline int wide_class_of(int Ee)
+// The class of a pair for the ring teams (up to ring_limit) or the index (E'
+// up to its largest).
+__host__ __device__ inline int wide_class_of(
+    int Ee, int ring_limit = ring_max_e(kRingClasses - 1))
 {
     int c = 0;
-    if (Ee <= ring_max_e(kRingClasses - 1)) {
+    if (Ee <= ring_limit) {
         while (Ee > ring_max_e(c))
             ++c;
         return kFirstRing + c;
@@ -104,16 +106,29 @@ __host__ __device__ inline int class_of(int m, int E)
 struct TuneParams {
     int rw_max_e = 31;
     int cw_subgrid = 8;
+    // largest E' a ring team takes (at most its classes' bound; the server's
+    // passes set a smaller one)
+    int ring_limit = ring_max_e(kRingClasses - 1);
 };
 
 __host__ __device__ inline int class_of_tuned(int m, int E,
                                               const TuneParams &tp)
 {
-    const int c = class_of(m, E);
-    // above the thread-per-pair limit: a team
-    if (c >= 0 && c < kRwClasses && eff_threshold(m, E) > tp.rw_max_e)
-        return wide_class_of(eff_threshold(m, E));
+    const int c = class_of(m, E), Ee = eff_threshold(m, E);
+    // above the thread-per-pair limit: a team; above the teams': the index
+    if (c >= 0 && c < kFirstIndex && Ee > tp.rw_max_e)
+        return wide_class_of(Ee, tp.ring_limit);
     return c;
+}
+
+// The serving engine's passes: pairs above 511 edits are long ones, which
+// leave their batch for the queue whose worker holds the index; in the
+// batch's class kernels they would hold its slot until the last is routed.
+__host__ __device__ inline TuneParams serving_params()
+{
+    TuneParams tp;
+    tp.ring_limit = 511;
+    return tp;
 }
 
 // Quarter-octave length bin, counted from the longest (bin 0) down.

@@ -1,4 +1,5 @@
-// ss_cwx.cuh -- K4 for thresholds from 817 to 10016: a CTA per pair, which
+// ss_cwx.cuh -- K4 for thresholds from 817 (in served batches 512) to 10016:
+// a CTA per pair, which
 // looks the longest escape segments up in an index of the query instead of
 // evaluating the maze rows.
 //

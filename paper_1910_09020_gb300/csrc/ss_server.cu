@@ -10,9 +10,8 @@
 // of the SMs, so that a batch admitted while others run executes beside
 // them instead of queueing behind them.
 //
-// Long pairs do not hold a slot.  The pairs of the index classes
-// (thresholds from 817 to 10016) go into a
-// device-resident ring instead of their batch's class kernels, and one
+// Long pairs do not hold a slot.  The pairs with thresholds from
+// 512 to 10016 go into a device-resident ring instead of their batch's class kernels, and one
 // long-lived persistent worker kernel (one CTA per SM)
 // drains that ring for every batch: a slot frees as soon as its pass ends,
 // while its long pairs run beside later batches' work.  The worker exits
@@ -269,8 +268,9 @@ __global__ void __launch_bounds__(ssk::kIndexThreads)
         if (!(bad && bad[p])) {
             const int64_t off = ps.off(p);
             count = ssk::index_route_any(
-                ssk::class_of(m, E) - ssk::kFirstIndex, smem, s,
-                ps.reads + off, ps.refs + off, m, E);
+                ssk::class_of_tuned(m, E, ssk::serving_params()) -
+                    ssk::kFirstIndex,
+                smem, s, ps.reads + off, ps.refs + off, m, E);
         }
         if (t == 0) {
             ps.acc[p] = (uint8_t)(count >= 0 && count <= E);
@@ -462,7 +462,7 @@ int launch_batch(ss_server *s, int slot_idx, std::vector<Request *> &take)
     int64_t nlong = 0;
     std::vector<int64_t> counts(ssk::kClasses, 0), queued(ssk::kClasses, 0);
     {
-        const ssk::TuneParams tp;
+        const ssk::TuneParams tp = ssk::serving_params();
         for (int64_t k = 0; k < n; ++k) {
             const int m = h_len[k], E = h_E[k];
             const int cls = ssk::class_of_tuned(m, E, tp);
@@ -498,9 +498,9 @@ int launch_batch(ss_server *s, int slot_idx, std::vector<Request *> &take)
         hp = &hook;
     }
     if (e == cudaSuccess)
-        e = ssk::launch_bucketed(ps, ssk::bucket_ws_at(ws, n), ssk::TuneParams(),
-                                 b->status, share, st, sl.side, sl.fork,
-                                 sl.join, false, &launches, hp,
+        e = ssk::launch_bucketed(ps, ssk::bucket_ws_at(ws, n),
+                                 ssk::serving_params(), b->status, share, st,
+                                 sl.side, sl.fork, sl.join, false, &launches, hp,
                                  hp ? (int)nlong : 0, counts.data());
     if (e == cudaSuccess) {
         const int g = (int)std::min<int64_t>((n + 255) / 256, 4 * s->sm_count);
