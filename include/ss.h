@@ -260,10 +260,10 @@ int ss_check_wait_timeout(ss_ctx *ctx, int64_t limit_ns, void *stream);
  * identical arguments; in the graph a class kernel runs only when its
  * class has pairs.  Two knobs change speed, never results:
  *   rw_max_e   15 or 31: largest E' routed with one thread per pair (above
- *              it, one warp or one CTA per pair, rows across the lanes);
+ *              it, a team of lanes or one CTA per pair);
  *   cw_subgrid 4, 8 or 16: columns evaluated across all rows per step by
- *              the warp/CTA kernels before surviving runs are extended
- *              32 columns at a time.
+ *              the CTA kernel of the largest thresholds before surviving
+ *              runs are extended 32 columns at a time.
  * ss_autotune() times every combination on the given batch (device
  * pointers as in ss_filter_batch, outputs written) and keeps the fastest in
  * the context; ss_set_tuning()/ss_get_tuning() set or read them directly.
@@ -299,8 +299,8 @@ int ss_filter_confusion(ss_ctx *ctx, const uint8_t *accept,
 /* ss_edit_distance_varlen: the same capped distance for pairs of per-pair
  * length lengths[p] (both sequences) at word offset offsets[p] of `reads`
  * and `refs` (SS_FMT_PACKED2, int64 word offsets, device arrays) and
- * per-pair threshold E[p] <= 511; one warp per pair, the band spread over
- * its lanes.  out_ed[p] = min(ED, E[p] + 1); a pair with E[p] > 511 gets -1
+ * per-pair threshold E[p] <= 511; a team of 8 or 32 lanes per pair over the
+ * diagonals that can still come back.  out_ed[p] = min(ED, E[p] + 1); a pair with E[p] > 511 gets -1
  * and SS_ERR_UNSUPPORTED from the next ss_sync, a negative length or
  * threshold -1 and SS_ERR_INVALID_ARG.  Asynchronous on `stream`.  Returns
  * SS_OK, SS_ERR_INVALID_ARG or SS_ERR_CUDA. */
