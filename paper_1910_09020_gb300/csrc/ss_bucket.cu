@@ -472,6 +472,7 @@ cudaError_t launch_cw_classes(const LaunchCfg &cfg, CwArgs a, int subgrid,
                               int sm_share, const ScanCond &c, Fan *fan,
                               cudaStream_t st, const int64_t *counts)
 {
+    a.sms = std::max(sm_share, 1);
     // the index classes first: the pairs that take longest from start to end
     for (int i = 0; i < kClasses - kFirstRing; ++i) {
         a.cls = i < kClasses - kFirstIndex ? kFirstIndex + i

@@ -144,6 +144,7 @@ struct CwArgs {
     BucketWs ws;
     int cls;
     uint32_t neg1 = 0xffffffffu;  // passed at run time (see rw_route)
+    int sms = 1;      // SMs the launch spans
     int queued = 0;   // skip the pairs the serving queue takes
 };
 

@@ -283,48 +283,6 @@ SS_HD int column_longest(const uint32_t *tabs, const uint32_t *q,
     return best | open;
 }
 
-// The run of the row starting at j from column c, at most lim bases: every
-// lane of a warp calls it (on the host, one lane does all).
-SS_HD int warp_run(const uint32_t *q, const uint32_t *r, int w16, int j,
-                   int c, int lim)
-{
-#ifdef __CUDA_ARCH__
-    const int lane = threadIdx.x & 31;
-    for (int at = 0;; at += 32 * 16) {
-        const int o = at + 16 * lane;
-        int k = 0;
-        if (o < lim) {
-            uint32_t qlo, qhi, rlo, rhi;
-            int qn, rn;
-            base_window(q, w16, j + o, qlo, qhi, qn);
-            base_window(r, w16, c + o, rlo, rhi, rn);
-            const uint32_t x = (qlo ^ rlo) | (qhi ^ rhi);
-            k = imin(x ? ffs32(x) - 1 : 16, 16);
-        }
-        const uint32_t stop = __ballot_sync(0xffffffffu, k < 16);
-        if (stop) {
-            const int f = __ffs((int)stop) - 1;
-            return imin(__shfl_sync(0xffffffffu, o + k, f), lim);
-        }
-    }
-#else
-    uint32_t rlo, rhi;
-    int rn;
-    base_window(r, w16, c, rlo, rhi, rn);
-    return index_run(q, r, w16, j, c, lim, rlo, rhi, rn, 0);
-#endif
-}
-
-// Maximum over the lanes of a warp (the host: its one lane).
-SS_HD int warp_max(int v)
-{
-#ifdef __CUDA_ARCH__
-    return __reduce_max_sync(0xffffffffu, v);
-#else
-    return v;
-#endif
-}
-
 // f(start) for every start in lo..hi whose K-mer is one of k0..k1, by lane
 // t of nt (four to a table), until f returns false.
 template <class Sh, class F>
