@@ -237,9 +237,9 @@ size_t cw_class_smem(int cls)
     default: break;
     }
     switch (cls - kFirstIndex) {
-    case 0: return IndexShape0::WORDS * 4;
-    case 1: return IndexShape1::WORDS * 4;
-    case 2: return IndexShape2::WORDS * 4;
+    case 0: return index_smem_words<0>() * 4;
+    case 1: return index_smem_words<1>() * 4;
+    case 2: return index_smem_words<2>() * 4;
     default: break;
     }
     const int M = cta_mbound(cls - kFirstCta);
@@ -473,11 +473,10 @@ cudaError_t launch_cw_classes(const LaunchCfg &cfg, CwArgs a, int subgrid,
                               cudaStream_t st, const int64_t *counts)
 {
     a.sms = std::max(sm_share, 1);
-    // the index classes first: the pairs that take longest from start to end
-    for (int i = 0; i < kClasses - kFirstRing; ++i) {
-        a.cls = i < kClasses - kFirstIndex ? kFirstIndex + i
-                                           : kFirstRing + i -
-                                                 (kClasses - kFirstIndex);
+    // from the largest thresholds down: the pairs that take longest from
+    // start to end first (1000 pairs of 10 to 100 kbp at 10 %, the other way
+    // round: 2.25 ms instead of 2.15)
+    for (a.cls = kClasses - 1; a.cls >= kFirstRing; --a.cls) {
         if (counts && counts[a.cls] == 0)
             continue;
         unsigned threads = 0;

@@ -1,7 +1,7 @@
 // ss_cwx.cuh -- K4 for thresholds from 817 (in served batches 512) to 10016:
-// a CTA per pair, which
-// looks the longest escape segments up in an index of the query instead of
-// evaluating the maze rows.
+// a CTA per pair, which looks the longest escape segments up in an index of
+// the query instead of evaluating the maze rows; where that does not pay, it
+// evaluates them.
 //
 // Method (Section 2.4): from checkpoint c the longest escape segment is the
 // longest match of R[c..] with the query from any start j in c-E..c+E.  At
@@ -17,12 +17,11 @@
 // instead of the latency of its lookups.  (One warp per pair walking the
 // chain lookup by lookup: 177 dependent instructions and 0.54 us a step; one
 // CTA of 512 threads evaluating all rows with a barrier per step: 0.7 to 1.2
-// us.)  What few columns need is done only where the chain stands on them,
-// by its warp:
-//   * a thread compares a start over at most kIndexWindows windows; the warp
-//     extends a longer run, 512 bases per comparison;
-//   * a column with several longer runs lies in a repeat: the warp compares
-//     all starts of its K-mer to the end;
+// us.)  What few columns need is done only where the chain stands on them:
+//   * a thread compares a start over at most kIndexWindows windows; the
+//     chain's warp extends a longer run, 512 bases per comparison;
+//   * a column with several longer runs, or with more starts than a thread
+//     is to go through, lies in a repeat: the CTA goes over to all rows;
 //   * a column whose K-mer has no start in reach has a run shorter than K.
 //     K-mers are numbered with the first base most significant, so the
 //     starts of a shorter prefix are those of consecutive K-mers.
@@ -216,9 +215,14 @@ SS_HD void table_scatter(uint32_t *tab, const uint32_t *q, int w16, int m,
 // A column's result: the longest run found, 0 if no start shares its K-mer
 // (the run is shorter than K); with kColumnOpen one start's run is not
 // known to its end, and its row j - c + Ee is at bits 8 and up;
-// kColumnRepeat: several starts' are not.
+// kColumnRepeat: several starts' are not; kColumnMany: more starts share the
+// K-mer, or agree with the column past it, than a thread looks at.
 constexpr int kColumnOpen = 1 << 29, kColumnRepeat = 1 << 30;
+constexpr int kColumnMany = kColumnRepeat + 1;
 constexpr int kIndexWindows = 3;  // 51 to 96 bases of a start
+// (random bases: two starts of a K-mer in a block at the most, five in reach,
+// one in 16 of which agrees in the next two, where these are known)
+constexpr int kIndexStarts = 24, kIndexExtends = 12;
 
 // Longest match of R[c..] among the starts c-Ee..c+Ee in the tables.
 template <class Sh>
@@ -235,6 +239,7 @@ SS_HD int column_longest(const uint32_t *tabs, const uint32_t *q,
     const uint32_t bases = bases_of_window(rlo, rhi);
     const uint32_t k = kmer_of<K>(bases), want = next_two<K>(bases);
     int best = 0, open = 0;
+    int extends = 0;
     int p0 = -1, p1 = -1;  // starts still to extend
     // (a start whose run is open: its row; false once there are two)
     auto extend = [&](int j) {
@@ -259,7 +264,10 @@ SS_HD int column_longest(const uint32_t *tabs, const uint32_t *q,
         const uint32_t mask =
             imax(c, base + Sh::BS - 1) + K + 2 > m ? 0u : 0xf000u;
         const int e = end[k];
-        for (int x = k ? end[k - 1] : 0; x < e; ++x) {
+        int x = k ? end[k - 1] : 0;
+        if (e - x > kIndexStarts)
+            return kColumnMany;
+        for (; x < e; ++x) {
             const uint32_t v = entry[x];
             const int j = base + (int)(v & 0xfffu);
             if ((uint32_t)(j - lo) > (uint32_t)(hi - lo))
@@ -271,6 +279,8 @@ SS_HD int column_longest(const uint32_t *tabs, const uint32_t *q,
                 p0 = j;
             } else if (p1 < 0) {
                 p1 = j;
+            } else if ((extends += mask ? 3 : 1) > kIndexExtends) {
+                return kColumnMany;
             } else if (!extend(j)) {
                 return kColumnRepeat;
             }
@@ -360,19 +370,22 @@ SS_HD int short_longest(const uint32_t *tabs, const uint32_t *q,
     return best;
 }
 
-// The chain's state.
+// The chain's state; done: 1 at its end, kChainMany on a column with too many
+// starts (if it stops there).
 struct IndexChain {
     int c, count, done;
 };
+constexpr int kChainMany = 2;
 
 // Follow the chain from s.c through the columns c0..c0+cols-1, whose
 // results are in col[] (all lanes of a warp, with the same state): one
-// obstacle after each run (Section 2.4 steps 3 and 4).
+// obstacle after each run (Section 2.4 steps 3 and 4).  many: stop at a column
+// with more starts than kIndexRepeat (else the warp compares all of them).
 template <class Sh>
 SS_HD void chain_follow(IndexChain &s, const int *col, int c0, int cols,
                         const uint32_t *tabs, const uint32_t *q,
                         const uint32_t *r, int w16, int m, int E, int Ee,
-                        int t, int nt)
+                        int t, int nt, bool many = false)
 {
     while (!s.done && s.c - c0 < cols) {
         const int v = col[s.c - c0];
@@ -380,7 +393,10 @@ SS_HD void chain_follow(IndexChain &s, const int *col, int c0, int cols,
         if (v & kColumnOpen) {
             const int j = ((v & (kColumnOpen - 1)) >> 8) - Ee + s.c;
             run = imax(run, warp_run(q, r, w16, j, s.c, m - imax(j, s.c)));
-        } else if (v == kColumnRepeat) {
+        } else if (v >= kColumnRepeat && many) {
+            s.done = kChainMany;
+            return;
+        } else if (v >= kColumnRepeat) {
             run = repeat_longest<Sh>(tabs, q, r, w16, m, Ee, s.c, t, nt);
         } else if (v == 0) {
             run = short_longest<Sh>(tabs, q, r, w16, m, Ee, s.c, t, nt);
@@ -396,6 +412,29 @@ SS_HD void chain_follow(IndexChain &s, const int *col, int c0, int cols,
     }
 }
 
+// ---- all rows ----------------------------------------------------------------
+//
+// What the index does not answer cheaply -- columns whose K-mer has many
+// starts, as in a repeat, and pairs whose steps are so long that most columns
+// looked up are never stood on -- the CTA routes by all rows (ss_cws.cuh), 32
+// to a thread, whatever the bases; then the index goes on.  Ms, the index
+// alone / with all rows / a CTA over all rows from the start, the whole pair
+// staged: 20 pairs of 10 to 100 kbp of a dinucleotide repeat with 5 % errors,
+// E = 10 %, 830 / 10.4 / 9.2; of a 171-base repeat 16.6 / 7.3 / 5.5; 1000 of
+// it of 10 to 30 kbp 3.7 / 2.1 / 2.1; 152 pairs of 100 kbp, E = 1 %, 0.8 %
+// errors 1.5 / 0.64 / 0.65, E = 10 %, 8 % errors 2.0 / 2.1 / 6.0.
+
+// The rings of a CTA of THREADS threads that takes one pair.
+template <int QB_, int RB_, int THREADS_>
+struct RowsShape {
+    static constexpr int QB = QB_, RB = RB_, BP = 1024, LANES = THREADS_;
+    static constexpr int QW = QB / 32, RW = RB / 32;
+    static constexpr int AHEAD = 32 * 32 + 95;  // a warp follows a row
+    static constexpr int WORDS = 2 * (QW + 1 + RW + 1);
+    static constexpr int max_e() { return (QB - BP - AHEAD - 1) / 2; }
+    static_assert(RB >= BP + AHEAD + 1, "a step in the reference's ring");
+};
+
 // The classes' shapes: one to five starts per K-mer and window.
 using IndexShape0 = IndexShape<5, 11, 3>;  // E' <= 1664:   18 KB
 using IndexShape1 = IndexShape<6, 12, 4>;  // E' <= 5920:   64 KB
@@ -406,21 +445,61 @@ static_assert(IndexShape0::max_e() >= index_max_e(0) &&
                   IndexShape2::max_e() >= index_max_e(2),
               "a class's thresholds fit its tables");
 
+// STEPS: as many steps by all rows take as long as a turn of kIndexCols columns
+// (a pair alone: 0.34 us each at E' = 1000, 0.6 at 5000, 1.2 at 10^4, against
+// 2.5, 3.0 and 4.0 a turn).
 template <int C>
 struct IndexClass;
 template <>
-struct IndexClass<0> { using Shape = IndexShape0; };
+struct IndexClass<0> {
+    using Shape = IndexShape0;
+    using Rows = RowsShape<16384, 8192, kIndexThreads>;
+    static constexpr int STEPS = 4;
+};
 template <>
-struct IndexClass<1> { using Shape = IndexShape1; };
+struct IndexClass<1> {
+    using Shape = IndexShape1;
+    using Rows = RowsShape<16384, 8192, kIndexThreads>;
+    static constexpr int STEPS = 3;
+};
 template <>
-struct IndexClass<2> { using Shape = IndexShape2; };
+struct IndexClass<2> {
+    using Shape = IndexShape2;
+    using Rows = RowsShape<32768, 8192, kIndexThreads>;
+    static constexpr int STEPS = 2;
+};
+
+// Shared words of a CTA of index class C: the tables, or in their place the
+// rings of all rows.  (Rings beside the tables would save building them again,
+// but left room for fewer CTAs on an SM: 1000 pairs of 10 to 100 kbp at 10 %
+// 2.15 -> 2.4 ms.)
+template <int C>
+constexpr int index_smem_words()
+{
+    static_assert(IndexClass<C>::Rows::max_e() >= index_max_e(C),
+                  "a class's thresholds fit its rings");
+    static_assert(IndexClass<C>::Rows::WORDS <= IndexClass<C>::Shape::WORDS,
+                  "the rings in the tables' place");
+    return IndexClass<C>::Shape::WORDS;
+}
+
+// Pairs whose obstacles, if they use up E, are on average more than this many
+// columns apart begin by all rows.
+constexpr int kIndexSparse = 32;
 
 #ifdef __CUDACC__
+constexpr int kRowsWarps = kIndexThreads / 32;
+struct RowsShared {
+    int best[2][kRowsWarps];
+    IndexChain chain;
+};
+
 // What the threads of a CTA share besides the tables.
 struct IndexShared {
     int col[2][kIndexCols];  // the columns' results
     uint32_t part[kIndexCols / 32];
     IndexChain chain;
+    RowsShared rows;
 };
 
 // Barrier of the kIndexCols threads that look columns up.
@@ -460,22 +539,139 @@ __device__ __forceinline__ void build_table(uint32_t *tab, IndexShared &s,
     cols_sync();
 }
 
-// Route one pair with the CTA's kIndexThreads threads; tabs: Sh::WORDS
-// words.  Returns min(count, E+1) to every thread.  Ee = eff_threshold(m,
-// E) <= max_e().
+// Barrier of the CTA's first n threads.
+__device__ __forceinline__ void rows_sync(int n)
+{
+    asm volatile("bar.sync 2, %0;" : : "r"(n) : "memory");
+}
+
+// Maximum over the first n threads of v, the same in the lanes of a warp
+// (best: a buffer their next call does not use).
+__device__ __forceinline__ int rows_best(int (&best)[kRowsWarps], int n, int v)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane == 0)
+        best[threadIdx.x >> 5] = v;
+    rows_sync(n);
+    return __reduce_max_sync(0xffffffffu, lane < n >> 5 ? best[lane] : 0);
+}
+
+// Follow the chain of a pair from s.c by all rows, until its end or until
+// the index would be faster: for `calm` stretches of kRowsStretch columns in
+// a row no lane had many survivors, and the last one's steps were of fewer
+// than `dense` columns each; x: Sh::WORDS words.  As many of the CTA's warps
+// take part as the window has words for.  (With half as many and two words a
+// lane 152 pairs of 100 kbp at E' = 1500 took 950 us instead of 790.)
+constexpr int kRowsStretch = 2048;
 template <class Sh>
-__device__ __noinline__ int index_route(uint32_t *tabs, IndexShared &s,
+__device__ __noinline__ void rows_route(uint32_t *x, RowsShared &sh,
+                                        IndexChain &chain, const uint32_t *q,
+                                        const uint32_t *r, int m, int E,
+                                        int Ee, int calm, int dense)
+{
+    const int t = threadIdx.x;
+    const int nt = min((2 * Ee + 1 + 1023) >> 10, Sh::LANES / 32) * 32;
+    if (t < nt) {
+        uint2 *q2 = reinterpret_cast<uint2 *>(x), *r2 = q2 + Sh::QW + 1;
+        RingStep s;
+        s.q2 = q2;
+        s.r2 = r2;
+        s.q = q;
+        s.r = r;
+        s.m = m;
+        s.w16 = (m + 15) >> 4;
+        s.c = chain.c;
+        int count = chain.count, qn = 0, rn = 0, buf = 0, quiet = 0;
+        bool over = false;
+        while (!over) {
+            // fill the rings as far as they go
+            qn = max(qn, max(s.c - Ee, 0) & ~(Sh::BP - 1));
+            rn = max(rn, s.c & ~(Sh::BP - 1));
+            const int q0 = qn, r0 = rn;
+            while (ring_room(qn, m, s.c - Ee, Sh::QB, Sh::BP))
+                qn += Sh::BP;
+            while (ring_room(rn, m, s.c, Sh::RB, Sh::BP))
+                rn += Sh::BP;
+            ring_fill<Sh::QW>(q2, q, s.w16, q0, qn, t, nt);
+            ring_fill<Sh::RW>(r2, r, s.w16, r0, rn, t, nt);
+            const int until = min(min(ring_until(qn, m, Ee + Sh::AHEAD),
+                                      ring_until(rn, m, Sh::AHEAD)),
+                                  s.c + kRowsStretch);
+            rows_sync(nt);
+            const int c0 = s.c, count0 = count;
+            bool many = false;
+            do {
+                ring_window<Sh::RW>(r2, s.c, s.rlo, s.rhi);
+                s.lo = max(s.c - Ee, 0);
+                s.hi = min(s.c + Ee, m - 1);
+                int best = rows_best(sh.best[buf], nt,
+                                     rows_step<Sh>(s, t, 32 * nt, many));
+                buf ^= 1;
+                if (best < 4) {
+                    int pre = 0;
+                    for (int i = (s.lo >> 5) + t; i <= s.hi >> 5; i += nt)
+                        pre = max(pre, prefix_word<Sh>(s, m - s.c, i));
+                    best = rows_best(sh.best[buf], nt, warp_max(pre));
+                    buf ^= 1;
+                }
+                s.c += best + 1;
+                count += s.c <= m ? 1 : 0;
+                over = s.c >= m || count > E;
+            } while (!over && s.c < until);
+            // (the barrier also lets the rings be written again)
+            const int any = rows_best(sh.best[buf], nt,
+                                      __any_sync(0xffffffffu, many));
+            buf ^= 1;
+            quiet = any ? 0 : quiet + 1;
+            if (quiet >= calm && s.c - c0 < dense * (count - count0))
+                over = true;
+        }
+        if (t == 0)
+            sh.chain = IndexChain{s.c, count, s.c >= m || count > E};
+    }
+    __syncthreads();
+    chain = sh.chain;
+    __syncthreads();  // sh.chain is written again
+}
+
+// Route one pair with the CTA's kIndexThreads threads; smem:
+// index_smem_words<C>() words.  Returns min(count, E+1) to every thread.
+// Ee = eff_threshold(m, E) <= max_e().
+template <int C>
+__device__ __noinline__ int index_route(uint32_t *smem, IndexShared &s,
                                         const uint32_t *q, const uint32_t *r,
                                         int m, int E)
 {
+    using Sh = typename IndexClass<C>::Shape;
+    using Rows = typename IndexClass<C>::Rows;
+    uint32_t *tabs = smem, *rings = smem;  // one or the other
     const int t = threadIdx.x;
     const int Ee = eff_threshold(m, E), w16 = (m + 15) >> 4;
+    constexpr int STEPS = IndexClass<C>::STEPS;
+    constexpr int DENSE = kIndexCols / (2 * STEPS);
     int built = 0, buf = 0;
+    int calm = 1;  // quiet stretches by all rows before the index goes on
+    int steps = 8 * STEPS;       // of the last turns, their mean four times
+    int before = 0;              // obstacles before a turn
     // columns at..: being looked up into col[buf]; those at c0..: in
     // col[buf ^ 1], for the chain (none in the first turn)
     int at = 0, c0 = -kIndexCols;
     IndexChain chain{0, 0, 0};
+    bool rows = (int64_t)Ee * kIndexSparse < m;
     for (;;) {
+        if (rows) {
+            rows_route<Rows>(rings, s.rows, chain, q, r, m, E, Ee, calm,
+                             DENSE);
+            if (chain.done)
+                return chain.count;
+            // (the columns looked up ahead are dropped, the tables built again)
+            rows = false;
+            built = 0;
+            steps = 8 * STEPS;
+            before = chain.count;
+            at = chain.c;
+            c0 = at - kIndexCols;
+        }
         if (t < kIndexCols) {
             const int last = min(at + kIndexCols - 1 + Ee, m - 1);
             // (blocks that a long run passed over are not built)
@@ -487,14 +683,26 @@ __device__ __noinline__ int index_route(uint32_t *tabs, IndexShared &s,
                 column_longest<Sh>(tabs, q, r, w16, m, Ee, at + t);
         } else {
             chain_follow<Sh>(chain, s.col[buf ^ 1], c0, kIndexCols, tabs, q,
-                             r, w16, m, E, Ee, t - kIndexCols, 32);
+                             r, w16, m, E, Ee, t - kIndexCols, 32, true);
             if (t == kIndexCols)
                 s.chain = chain;
         }
         __syncthreads();
         chain = s.chain;
-        if (chain.done)
+        if (chain.done == 1)
             return chain.count;
+        if (chain.done == kChainMany) {
+            // a repeat: by all rows until it is over, longer each time
+            chain.done = 0;
+            calm = min(2 * calm, 64);
+            rows = true;
+            continue;
+        }
+        // steps so long that most columns are looked up in vain
+        if (c0 >= 0)
+            steps += chain.count - before - (steps >> 2);
+        before = chain.count;
+        rows = steps < 4 * STEPS;
         c0 = at;
         // the chain may have left these columns behind already
         at = max(at + kIndexCols, chain.c);
@@ -504,25 +712,25 @@ __device__ __noinline__ int index_route(uint32_t *tabs, IndexShared &s,
 }
 
 // Route a pair of index class ic.
-__device__ __forceinline__ int index_route_any(int ic, uint32_t *tabs,
+__device__ __forceinline__ int index_route_any(int ic, uint32_t *smem,
                                                IndexShared &s,
                                                const uint32_t *q,
                                                const uint32_t *r, int m,
                                                int E)
 {
     switch (ic) {
-    case 0: return index_route<IndexShape0>(tabs, s, q, r, m, E);
-    case 1: return index_route<IndexShape1>(tabs, s, q, r, m, E);
-    default: return index_route<IndexShape2>(tabs, s, q, r, m, E);
+    case 0: return index_route<0>(smem, s, q, r, m, E);
+    case 1: return index_route<1>(smem, s, q, r, m, E);
+    default: return index_route<2>(smem, s, q, r, m, E);
     }
 }
 
 // A pair at a time from the class's queue.
 template <int C>
-__global__ void __launch_bounds__(kIndexThreads) k_cw_index(const CwArgs a)
+__global__ void __launch_bounds__(kIndexThreads, C == 0 ? 4 : 3)
+    k_cw_index(const CwArgs a)
 {
-    using Sh = typename IndexClass<C>::Shape;
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     __shared__ IndexShared s;
     __shared__ int s_idx;
     const int t = threadIdx.x;
@@ -530,22 +738,22 @@ __global__ void __launch_bounds__(kIndexThreads) k_cw_index(const CwArgs a)
     const int end = a.ws.ranges[2 * a.cls + 1];
     if (a.queued && long_queued(a.cls))
         return;  // routed by the serving queue's worker
-    for (;;) {
-        if (t == 0)
-            s_idx = begin + (int)atomicAdd(&a.ws.counters[a.cls], 1u);
-        __syncthreads();
-        const int idx = s_idx;
-        if (idx >= end)
-            break;
+    // the first without waiting for the counter (in the order of their
+    // claims, few pairs stood two on every other SM)
+    for (int idx = begin + (int)blockIdx.x; idx < end;) {
         const int64_t p = a.ws.perm[idx];
         const int m = a.ps.len(p), E = a.ps.thr(p);
         const int64_t off = a.ps.off(p);
-        const int count = index_route<Sh>(smem, s, a.ps.reads + off,
-                                          a.ps.refs + off, m, E);
+        const int count = index_route<C>(smem, s, a.ps.reads + off,
+                                         a.ps.refs + off, m, E);
         if (t == 0) {
             a.ps.acc[p] = (uint8_t)(count <= E);
             a.ps.obs[p] = count;
+            s_idx = begin + (int)gridDim.x +
+                    (int)atomicAdd(&a.ws.counters[a.cls], 1u);
         }
+        __syncthreads();
+        idx = s_idx;
         __syncthreads();  // the tables and s_idx are reused
     }
 }

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(ssk::kIndexThreads)
     }
 }
 
-size_t worker_smem() { return (size_t)ssk::IndexShape2::WORDS * 4; }
+size_t worker_smem() { return (size_t)ssk::index_smem_words<2>() * 4; }
 
 // Launch the worker if work is in flight (want, or queued pairs remain)
 // and none is running.  It is launched ahead of each batch's kernels: its

@@ -79,6 +79,68 @@ def check(F, cases, seed, what, flags=0):
     return oacc
 
 
+BOUNDS = [32, 112, 113, 304, 305, 511, 512, 816, 817, 1664, 1665, 5920, 5921,
+          10016, 10017]
+
+
+@pytest.mark.parametrize("flags", [0, binding.SS_FLAG_NO_GRAPH])
+def test_class_bounds(F, flags):
+    """Thresholds either side of every class bound, lengths around the words
+    and rings and far above the threshold, accurate and rejected pairs, and
+    thresholds above the length."""
+    cases = []
+    for e in BOUNDS:
+        for m in sorted({e + 1, e + 2, e + 33, 2 * e + 5, 16384, 16385}):
+            if m <= e:
+                continue
+            for rate in (0.01, 0.25):
+                cases.append((0, m, rate, e))
+    for m in (33, 113, 305, 817, 1665, 5921, 10017, 10018):
+        cases.append((0, m, 0.3, m + 7))       # clamped to m - 1
+    cases += [(0, 65536, 0.02, 3000), (0, 65537, 0.06, 7000),
+              (0, 131072, 0.05, 10016), (0, 131072, 0.12, 10017),
+              (0, 131072, 0.003, 500), (0, 131072, 0.01, 2000),
+              (0, 131072, 0.1, 131071)]
+    acc = check(F, cases, 3, "class bounds", flags)
+    assert 0 < acc.mean() < 1
+
+
+@pytest.mark.parametrize("kind", [1, 2, 3, 4])
+def test_repeats(F, kind):
+    """Repeats through every class above 31 edits: the index leaves them to
+    all rows and, after the repeat of kind 4, goes on."""
+    cases = [(kind, m, rate, e)
+             for e in (40, 112, 300, 500, 816, 900, 1664, 3000, 8000, 12000)
+             for m in (e + 40, 3 * e, 12 * e) if m < 60000
+             for rate in (0.0, 0.02, 0.2)]
+    check(F, cases, 10 + kind, f"repeats, kind {kind}")
+
+
+def test_accurate_and_changing_pairs(F):
+    """Long pairs whose steps are long (all rows) or short (the index), and
+    pairs whose error rate changes on the way."""
+    cases = [(0, m, rate, m * pm // 1000) for m in (30000, 100000)
+             for rate in (0.0, 0.001, 0.01, 0.03, 0.15)
+             for pm in (10, 20, 50, 100)]
+    check(F, cases, 20, "accurate pairs")
+    torch = torch_cuda()
+    rng = np.random.default_rng(21)
+    letters = np.frombuffer(b"ACGT", np.uint8)
+    for e in (1500, 4000, 9000):
+        q = rng.integers(0, 4, 10 * e)
+        parts = [noisy(rng, x, rate) for x, rate in
+                 zip(np.array_split(q, 6), (.005, .12, .01, .1, .002, .15))]
+        r = np.concatenate(parts)
+        qa, ra = letters[q], letters[r]
+        m = len(q)
+        dq, dr = (F.pack(to_dev(x), m=m, n=1) for x in (qa, ra))
+        acc, obs = F.filter(dq, dr, m=m, e=e, n=1, sync=True)
+        want = oracle.filter_pair(qa.tobytes(), ra.tobytes(), e)
+        assert int(obs[0]) == want.obstacles
+        assert bool(acc[0]) == want.accept
+    torch.cuda.synchronize()
+
+
 @pytest.mark.parametrize("m,e", [(400, 40), (700, 112), (900, 200),
                                  (1200, 310), (1500, 600)])
 @pytest.mark.parametrize("n", [60, 3000, 30000])
@@ -99,3 +161,17 @@ def test_few_and_many_pairs(F, m, e, n):
     acc, obs = F.filter(q, r, m=m, e=e, n=n, sync=True)
     assert_same(acc.cpu().numpy(), obs.cpu().numpy(), oacc[pick], oobs[pick],
                 f"n={n} m={m} e={e}")
+
+
+@pytest.mark.parametrize("k", [4, 8, 16])
+def test_subgrids_of_the_largest_thresholds(F, k):
+    """Every subgrid of the CTA kernel, which only pairs above 10016 edits
+    reach, in every length bound of its classes."""
+    F.set_tuning(31, k)
+    try:
+        check(F, [(kind, m, rate, e) for kind in (0, 2)
+                  for m, e in ((10050, 10020), (16384, 12000), (16385, 16384),
+                               (40000, 11000), (65537, 10017))
+                  for rate in (0.02, 0.3)], 40, f"subgrid {k}")
+    finally:
+        F.set_tuning(31, 8)

@@ -1,5 +1,6 @@
-"""Host builds of the routes above 31 edits that do not depend on the bases
-(all rows of a pair), against the oracle, and of what leads to them."""
+"""Host builds of the routes above 31 edits that do not depend on the bases:
+a warp or a CTA per pair over all rows, and the index' way into them on
+repeats and back, against the oracle."""
 import ctypes
 import os
 import subprocess
@@ -38,6 +39,8 @@ def emu():
     lib = ctypes.CDLL(out)
     P, I = ctypes.c_void_p, ctypes.c_int
     lib.emu_rows.argtypes = [P, P, I, I, I]
+    lib.emu_index_rows.argtypes = [P, P, I, I, I, I, P]
+    lib.emu_column.argtypes = [P, P, I, I, I]
     lib.emu_rows_max_e.argtypes = [I]
     lib.emu_handed_over.argtypes = [P, P, I, I]
     lib.emu_first_pair.argtypes = [I, I, I]
@@ -94,7 +97,7 @@ def plain(seed, m):
     return out
 
 
-@pytest.mark.parametrize("which", [0])
+@pytest.mark.parametrize("which", [0, 1, 2, 3])
 def test_all_rows_match_oracle(emu, which):
     """Lengths around the words, the blocks of 1024 bases and the rings,
     thresholds from 0 to the largest of the rings."""
@@ -115,6 +118,37 @@ def test_all_rows_match_oracle(emu, which):
                 want = oracle.filter_pair(q, r, E).obstacles
                 got = emu.emu_rows(ptr(qw), ptr(rw), m, E, which)
                 assert got == want, (which, m, E, k)
+
+
+@pytest.mark.parametrize("ic,E", [(0, 817), (0, 1664), (1, 1665), (2, 6000)])
+@pytest.mark.parametrize("calm", [1, 8])
+def test_index_leaves_repeats_to_all_rows(emu, ic, E, calm):
+    """The index route of a repeat goes over to all rows and, between random
+    bases, comes back; the results are the oracle's."""
+    m = {0: 6000, 1: 9000, 2: 14000}[ic]
+    for k, (q, r) in enumerate(repeats(E, m) + plain(E, m)[2:3]):
+        if ic == 2 and k in (0, 4):
+            continue
+        qw, rw = packed(q), packed(r)
+        turns = ctypes.c_int()
+        got = emu.emu_index_rows(ptr(qw), ptr(rw), m, E, ic, calm,
+                                 ctypes.byref(turns))
+        assert got == oracle.filter_pair(q, r, E).obstacles, (ic, E, k)
+        if k in (0, 1, 3):
+            assert turns.value > 0
+        if k == 4 and got > 500:
+            assert turns.value == 0
+
+
+def test_index_thread_does_not_go_through_a_repeat(emu):
+    """A column of a repeat is left to all rows (its thousands of starts are
+    not gone through by one thread); one of random bases is not."""
+    m, E = 4000, 1600
+    for k, (q, r) in enumerate(repeats(5, m)[:2] + plain(6, m)[1:2]):
+        qw, rw = packed(q), packed(r)
+        many = [emu.emu_column(ptr(qw), ptr(rw), m, E, c)
+                for c in range(1900, 2100)]
+        assert (sum(many) > 100) if k < 2 else (sum(many) == 0)
 
 
 def test_teams_hand_repeats_over_to_their_warp(emu):
