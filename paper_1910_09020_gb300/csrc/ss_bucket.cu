@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256)
         s_n = 0;
     __syncthreads();
     int mine = 0;
-    for (int cls = kFirstIndex; cls < kFirstCta; ++cls) {
+    for (int cls = kFirstIndex; cls < kClasses; ++cls) {
         const int begin = ws.ranges[2 * cls], end = ws.ranges[2 * cls + 1];
         for (int i = begin + (int)threadIdx.x; i < end; i += blockDim.x) {
             const int64_t p = ws.perm[i];

@@ -220,10 +220,13 @@ constexpr int kLongBatches = 64;     // descriptors
 // beside the worker they waited for it to leave).
 constexpr int kLongCtasPerSm = 1;
 
-// Whether the queue takes the pairs of class cls: the index classes.
+// Whether the queue takes the pairs of class cls: the index and the CTA
+// classes.  (A batch's own CTA kernel takes up to 180 KB of an SM's shared
+// memory for a long pair: it would wait for the worker to leave, and hold the
+// batch's slot until then.)
 __host__ __device__ inline bool long_queued(int cls)
 {
-    return cls >= kFirstIndex && cls < kFirstCta;
+    return cls >= kFirstIndex;
 }
 
 // A batch's hook into the queue: its descriptor index, passed to the

@@ -196,6 +196,8 @@ __global__ void __launch_bounds__(1024) k_cw_cta(const CwArgs a)
     const int t = threadIdx.x;
     const int begin = a.ws.ranges[2 * a.cls];
     const int end = a.ws.ranges[2 * a.cls + 1];
+    if (a.queued && long_queued(a.cls))
+        return;  // routed by the serving queue's worker
     int buf = 0;
     for (;;) {
         if (t == 0)

@@ -711,7 +711,12 @@ __device__ __noinline__ int index_route(uint32_t *smem, IndexShared &s,
     }
 }
 
-// Route a pair of index class ic.
+// Route a pair of index class ic, or (above them) of any threshold: by all
+// rows, the whole query in the ring.
+using WholeRows = RowsShape<131072, 8192, kIndexThreads>;
+static_assert(WholeRows::QB >= kMaxLen &&
+                  WholeRows::WORDS <= index_smem_words<2>(),
+              "the longest query in the ring, in the tables' place");
 __device__ __forceinline__ int index_route_any(int ic, uint32_t *smem,
                                                IndexShared &s,
                                                const uint32_t *q,
@@ -721,8 +726,13 @@ __device__ __forceinline__ int index_route_any(int ic, uint32_t *smem,
     switch (ic) {
     case 0: return index_route<0>(smem, s, q, r, m, E);
     case 1: return index_route<1>(smem, s, q, r, m, E);
-    default: return index_route<2>(smem, s, q, r, m, E);
+    case 2: return index_route<2>(smem, s, q, r, m, E);
+    default: break;
     }
+    IndexChain chain{0, 0, 0};
+    rows_route<WholeRows>(smem, s.rows, chain, q, r, m, E,
+                          eff_threshold(m, E), 1, 0);
+    return chain.count;
 }
 
 // A pair at a time from the class's queue.

@@ -10,11 +10,11 @@
 // of the SMs, so that a batch admitted while others run executes beside
 // them instead of queueing behind them.
 //
-// Long pairs do not hold a slot.  The pairs with thresholds from
-// 512 to 10016 go into a device-resident ring instead of their batch's class kernels, and one
-// long-lived persistent worker kernel (one CTA per SM)
-// drains that ring for every batch: a slot frees as soon as its pass ends,
-// while its long pairs run beside later batches' work.  The worker exits
+// Long pairs do not hold a slot.  The pairs with thresholds above 511 go into
+// a device-resident ring instead of their batch's class kernels, and one
+// long-lived persistent worker kernel (one CTA per SM) drains that ring for
+// every batch: a slot frees as soon as its pass ends, while its long pairs
+// run beside later batches' work.  The worker exits
 // after a bounded idle time (or when the server stops) and the scheduler
 // relaunches it while queued pairs remain; its waits on the ring are
 // bounded.  A batch is done when its pass has ended (a host-function
@@ -238,11 +238,11 @@ __device__ int long_claim(const ssk::LongQueue &q, uint64_t idle_ns,
 }
 
 // The long-lived worker: each CTA takes queued pairs one at a time and
-// routes each (Section 2.4, by the index of ss_cwx.cuh); the CTA that routes
+// routes each (Section 2.4, as ss_cwx.cuh does); the CTA that routes
 // a batch's last queued pair publishes the batch's generation to the host.
 // Pairs flagged as holding a non-base get obstacles -1 (their batch's
 // request fails alone, as in the pass).
-__global__ void __launch_bounds__(ssk::kIndexThreads)
+__global__ void __launch_bounds__(ssk::kIndexThreads, 3)
     k_long_worker(const ssk::LongQueue q, uint64_t idle_ns)
 {
     extern __shared__ uint32_t smem[];

@@ -209,7 +209,9 @@ int emu_rows(const uint32_t *q, const uint32_t *r, int m, int E, int which)
     case 0: return all_rows<WarpShape>(q, r, m, E);
     case 1: return all_rows<IndexClass<0>::Rows>(q, r, m, E);
     case 2: return all_rows<IndexClass<1>::Rows>(q, r, m, E);
-    default: return all_rows<IndexClass<2>::Rows>(q, r, m, E);
+    case 3: return all_rows<IndexClass<2>::Rows>(q, r, m, E);
+    default: return all_rows<RowsShape<131072, 8192, kIndexThreads>>(q, r, m,
+                                                                     E);
     }
 }
 
@@ -239,6 +241,13 @@ int emu_column(const uint32_t *q, const uint32_t *r, int m, int E, int c)
         table_scatter<Sh>(tab, q, w16, m, b, 0, 1);
     }
     return column_longest<Sh>(tabs.data(), q, r, w16, m, Ee, c) == kColumnMany;
+}
+
+// Whether the serving queue takes a pair.
+int emu_long_queued(int m, int E)
+{
+    const int c = class_of_tuned(m, E, serving_params());
+    return c >= 0 && long_queued(c);
 }
 
 int emu_handed_over(const uint32_t *q, const uint32_t *r, int m, int E)

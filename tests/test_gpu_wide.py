@@ -175,3 +175,40 @@ def test_subgrids_of_the_largest_thresholds(F, k):
                   for rate in (0.02, 0.3)], 40, f"subgrid {k}")
     finally:
         F.set_tuning(31, 8)
+
+
+def test_served_pairs_above_the_index(F):
+    """Requests with pairs above 10016 edits, up to the longest, among a
+    stream of ordinary queued pairs: all of them go to the queue, and the
+    results are the oracle's."""
+    rng = np.random.default_rng(60)
+    letters = np.frombuffer(b"ACGT", np.uint8)
+    reqs = []
+    for k in range(8):
+        cases = [(0, m, 0.05, m // 10)
+                 for m in rng.integers(6000, 30000, 12)]
+        cases += [(0, int(m), 0.1, 60) for m in rng.integers(200, 4000, 12)]
+        if k % 2 == 0:
+            cases += [(0, 50000, 0.1, 12000), (2, 30000, 0.02, 11000),
+                      (0, 20000, 0.4, 19999)]
+        if k == 2:
+            cases += [(0, 131072, 0.12, 10017), (0, 70000, 0.02, 30000)]
+        sides = [pair(rng, c, int(m), rate) for c, m, rate, _ in cases]
+        L = np.array([c[1] for c in cases], np.int32)
+        E = np.array([c[3] for c in cases], np.int32)
+        off = np.concatenate([[0], np.cumsum(L, dtype=np.int64)])
+        reqs.append([letters[np.concatenate([s[i] for s in sides])]
+                     for i in (0, 1)] + [L, E, off])
+    queued = sum(int((np.minimum(r[3], r[2] - 1) > 511).sum()) for r in reqs)
+    with binding.Server(0, hbm_budget_bytes=4 << 30, slots=2) as S:
+        tickets = [S.submit(*r[:4]) for r in reqs]
+        outs = []
+        for t in tickets:
+            assert S.wait(t, timeout_s=60.0) == binding.SS_OK
+            outs.append(S.fetch(t))
+        stats = S.stats()
+    assert stats["long_pairs_queued"] == queued
+    for (rc, a, o, _), r in zip(outs, reqs):
+        assert rc == binding.SS_OK
+        oa, oo = oracle.filter_batch(r[0], r[1], r[2], r[3], offsets=r[4])
+        assert_same(a, o, oa, oo, "served")

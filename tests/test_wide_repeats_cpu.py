@@ -44,6 +44,7 @@ def emu():
     lib.emu_rows_max_e.argtypes = [I]
     lib.emu_handed_over.argtypes = [P, P, I, I]
     lib.emu_first_pair.argtypes = [I, I, I]
+    lib.emu_long_queued.argtypes = [I, I]
     return lib
 
 
@@ -149,6 +150,20 @@ def test_index_thread_does_not_go_through_a_repeat(emu):
         many = [emu.emu_column(ptr(qw), ptr(rw), m, E, c)
                 for c in range(1900, 2100)]
         assert (sum(many) > 100) if k < 2 else (sum(many) == 0)
+
+
+def test_queue_takes_every_pair_above_511_edits(emu):
+    """Also those above the index' thresholds, which would hold their batch's
+    slot until the worker has left; and a worker's route for them."""
+    for m in (600, 12000, 50000, 131072):
+        for E in (31, 511, 512, 5920, 10016, 10017, 12000, 65000, 131071):
+            e = min(E, m - 1)
+            assert emu.emu_long_queued(m, E) == (e > 511), (m, E)
+    for m, E in ((10100, 10017), (11000, 10999), (12000, 20000)):
+        for q, r in repeats(m, m)[:1] + plain(m, m)[:2]:
+            want = oracle.filter_pair(q, r, E).obstacles
+            qw, rw = packed(q), packed(r)
+            assert emu.emu_rows(ptr(qw), ptr(rw), m, E, 4) == want
 
 
 def test_teams_hand_repeats_over_to_their_warp(emu):
