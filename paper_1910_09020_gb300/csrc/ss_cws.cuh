@@ -41,13 +41,19 @@
 
 namespace ssk {
 
+// A packed word of a sequence, by an ordinary load: the serving queue's worker
+// runs these routes while other kernels write the sequences of later pairs,
+// and the read-only path (ldg) is for memory that no one writes during the
+// kernel.
+SS_HD uint32_t seq_word(const uint32_t *p) { return *p; }
+
 // Code bits of the 17 to 32 bases a sequence's words hold from base j on
 // (the number in n): bit t of lo/hi is base j + t.
 SS_HD void base_window(const uint32_t *g, int w16, int j, uint32_t &lo,
                        uint32_t &hi, int &n)
 {
     const int i = j >> 4, s = j & 15;
-    const uint32_t a = ldg(g + i), b = i + 1 < w16 ? ldg(g + i + 1) : 0u;
+    const uint32_t a = seq_word(g + i), b = i + 1 < w16 ? seq_word(g + i + 1) : 0u;
     lo = prmt(a, b, 0x5410u) >> s;
     hi = prmt(a, b, 0x7632u) >> s;
     n = 32 - s;
@@ -58,8 +64,8 @@ SS_HD void full_window(const uint32_t *g, int w16, int j, uint32_t &lo,
                        uint32_t &hi)
 {
     const int i = j >> 4;
-    const uint32_t a = ldg(g + i), b = i + 1 < w16 ? ldg(g + i + 1) : 0u;
-    const uint32_t z = i + 2 < w16 ? ldg(g + i + 2) : 0u;
+    const uint32_t a = seq_word(g + i), b = i + 1 < w16 ? seq_word(g + i + 1) : 0u;
+    const uint32_t z = i + 2 < w16 ? seq_word(g + i + 2) : 0u;
     lo = funnel_r(prmt(a, b, 0x5410u), z & 0xffffu, (uint32_t)j & 15u);
     hi = funnel_r(prmt(a, b, 0x7632u), z >> 16, (uint32_t)j & 15u);
 }
@@ -132,8 +138,8 @@ SS_HD void ring_load(uint2 *x, const uint32_t *g, int w16, int n, int t,
 #pragma unroll
     for (int k = 0; k < BP / 32; k += nt) {
         const int i = (n >> 5) + k + t, at = i & (W - 1);
-        const uint32_t a = 2 * i < w16 ? ldg(g + 2 * i) : 0u;
-        const uint32_t b = 2 * i + 1 < w16 ? ldg(g + 2 * i + 1) : 0u;
+        const uint32_t a = 2 * i < w16 ? seq_word(g + 2 * i) : 0u;
+        const uint32_t b = 2 * i + 1 < w16 ? seq_word(g + 2 * i + 1) : 0u;
         const uint2 v =
             make_uint2(prmt(a, b, 0x5410u), prmt(a, b, 0x7632u));
         x[at] = v;
@@ -149,8 +155,8 @@ SS_HD void ring_fill(uint2 *x, const uint32_t *g, int w16, int n0, int n1,
 {
     for (int i = (n0 >> 5) + t; i < n1 >> 5; i += nt) {
         const int at = i & (W - 1);
-        const uint32_t a = 2 * i < w16 ? ldg(g + 2 * i) : 0u;
-        const uint32_t b = 2 * i + 1 < w16 ? ldg(g + 2 * i + 1) : 0u;
+        const uint32_t a = 2 * i < w16 ? seq_word(g + 2 * i) : 0u;
+        const uint32_t b = 2 * i + 1 < w16 ? seq_word(g + 2 * i + 1) : 0u;
         const uint2 v =
             make_uint2(prmt(a, b, 0x5410u), prmt(a, b, 0x7632u));
         x[at] = v;

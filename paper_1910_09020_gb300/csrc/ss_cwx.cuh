@@ -141,8 +141,8 @@ SS_HD void block_starts(const uint32_t *q, int w16, int m, int b, int t,
     const int j1 = imin(j0 + Sh::BS, m - Sh::K + 1);
     for (int j = j0 + 16 * t; j < j1; j += 16 * nt) {
         const int i = j >> 4;  // j is a multiple of 16
-        const uint32_t a = bases_of_word(ldg(q + i));
-        const uint32_t z = i + 1 < w16 ? bases_of_word(ldg(q + i + 1)) : 0u;
+        const uint32_t a = bases_of_word(seq_word(q + i));
+        const uint32_t z = i + 1 < w16 ? bases_of_word(seq_word(q + i + 1)) : 0u;
 #pragma unroll
         for (int x = 0; x < 16; ++x)
             if (j + x < j1)

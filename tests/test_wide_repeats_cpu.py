@@ -187,3 +187,13 @@ def test_first_pairs_are_dealt_once(emu, grid, sms):
         first = [b for b in range(grid) if got[b] < sms]
         assert max(sum(b // sms == k for b in first)
                    for k in range(grid // sms)) <= sms // 8
+
+
+def test_worker_reads_sequences_by_ordinary_loads():
+    """The serving worker outlives the kernels that write its pairs'
+    sequences: its routes may not read them by the read-only path, which is
+    defined only for memory that does not change while a kernel runs."""
+    for name in ("ss_cws.cuh", "ss_cwx.cuh", "ss_server.cu"):
+        with open(os.path.join(CSRC, name)) as f:
+            code = "\n".join(line.split("//")[0] for line in f)
+        assert "ldg(" not in code and ".nc" not in code, name
