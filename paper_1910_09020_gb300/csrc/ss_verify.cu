@@ -137,22 +137,18 @@ __global__ void __launch_bounds__(32 * kEdVarWarps)
         __syncwarp();
         for (int e = 0;; ++e) {
             if (act) {
-                const bool there = F[e & 1][H + 1] >= m;
-                if (there || e == E) {
+                int ed;
+                if (ed_ends(F[e & 1][H + 1], m, E, e, ed)) {
                     if (tl == 0)
-                        a.ed[p] = there ? e : E + 1;
+                        a.ed[p] = ed;
                     act = false;
                 }
             }
             if (!__any_sync(0xffffffffu, act))
                 break;
-            if (act) {
-                const int w = min(e + 1, E - e - 1);
-                const int *prev = F[e & 1] + H + 1;
-                int *next = F[(e + 1) & 1] + H + 1;
-                for (int k = tl - w; k <= w; k += TEAM)
-                    next[k] = ed_diagonal(q, r, w16, m, prev + k, k);
-            }
+            if (act)
+                ed_advance(q, r, w16, m, E, e, F[e & 1] + H + 1,
+                           F[(e + 1) & 1] + H + 1, tl, TEAM);
             __syncwarp();
         }
         __syncwarp();  // F is reused by the next pair

@@ -60,6 +60,26 @@ SS_HD int ed_diagonal(const uint32_t *q, const uint32_t *r, int w16, int m,
     return t + ed_slide(q, r, w16, t, t + k, lim - t);
 }
 
+// Whether edit count e is the pair's last one: its distance in ed then
+// (at = F_e[0]).
+SS_HD bool ed_ends(int at, int m, int E, int e, int &ed)
+{
+    const bool there = at >= m;
+    ed = there ? e : E + 1;
+    return there || e == E;
+}
+
+// F_{e+1} (next) from F_e (prev, both at diagonal 0; e < E), by lane t of a
+// team of nt; what lies outside |k| <= min(e, E - e) of prev is kEdNone or
+// an older value, which is no further.
+SS_HD void ed_advance(const uint32_t *q, const uint32_t *r, int w16, int m,
+                      int E, int e, const int *prev, int *next, int t, int nt)
+{
+    const int w = imin(e + 1, E - e - 1);
+    for (int k = t - w; k <= w; k += nt)
+        next[k] = ed_diagonal(q, r, w16, m, prev + k, k);
+}
+
 // min(ED, E+1) of one pair, its diagonals one after another.
 template <int E>
 SS_HD int ed_banded(const uint32_t *q, const uint32_t *r, int m, int w16)
