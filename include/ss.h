@@ -264,7 +264,7 @@ int ss_check_wait_timeout(ss_ctx *ctx, int64_t limit_ns, void *stream);
  *   cw_subgrid 4, 8 or 16: columns evaluated across all rows per step by
  *              the CTA kernel of the largest thresholds before surviving
  *              runs are extended 32 columns at a time.
- * ss_autotune() times every combination on the given batch (device
+ * ss_autotune() times every combination that concerns the given batch (device
  * pointers as in ss_filter_batch, outputs written) and keeps the fastest in
  * the context; ss_set_tuning()/ss_get_tuning() set or read them directly.
  * Returns SS_OK, SS_ERR_INVALID_ARG, SS_ERR_OOM or SS_ERR_CUDA; best_ms

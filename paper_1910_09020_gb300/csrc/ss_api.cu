@@ -1464,8 +1464,13 @@ int ss_autotune(ss_ctx *ctx, const void *reads, const void *refs,
     SS_CUDA(cudaEventCreate(&a));
     SS_CUDA(cudaEventCreate(&z));
     int rc = SS_OK;
+    // the subgrids reach only the CTA classes: without pairs there (known
+    // after the first pass) the default stands
+    bool subgrids = true;
     for (int rmax : {15, 31}) {
-        for (int k : {4, 8, 16}) {
+        for (int k : {8, 4, 16}) {
+            if (k != 8 && !subgrids)
+                continue;
             ctx->tune.rw_max_e = rmax;
             ctx->tune.cw_subgrid = k;
             rc = run_bucketed(ctx, ps, st, false);  // warm-up
@@ -1479,6 +1484,18 @@ int ss_autotune(ss_ctx *ctx, const void *reads, const void *refs,
                 if (rc == SS_OK)
                     rc = SS_ERR_CUDA;
                 break;
+            }
+            if (k == 8) {
+                int range[2 * ssk::kCtaClasses];
+                if (cudaMemcpy(range,
+                               ssk::bucket_ws_at(ctx->ws, n).ranges +
+                                   2 * ssk::kFirstCta,
+                               sizeof range, cudaMemcpyDeviceToHost) !=
+                    cudaSuccess) {
+                    rc = SS_ERR_CUDA;
+                    break;
+                }
+                subgrids = range[2 * ssk::kCtaClasses - 1] > range[0];
             }
             float ms = 0;
             cudaEventElapsedTime(&ms, a, z);

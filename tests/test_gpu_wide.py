@@ -212,3 +212,20 @@ def test_served_pairs_above_the_index(F):
         assert rc == binding.SS_OK
         oa, oo = oracle.filter_batch(r[0], r[1], r[2], r[3], offsets=r[4])
         assert_same(a, o, oa, oo, "served")
+
+
+def test_autotune_leaves_subgrids_that_nothing_reaches(F):
+    """Without pairs above 10016 edits the subgrids do nothing: they are not
+    timed (a third of the passes) and the default stays."""
+    def passes(cases):
+        host, off, L, Es, dev, dwoff, dL = batch(F, cases, 70)
+        before = F.counters().launches
+        _, k, _ = F.autotune(dev[0], dev[1], offsets=dwoff, lengths=dL,
+                             E=to_dev(Es), reps=1)
+        return F.counters().launches - before, k
+    try:
+        few, k = passes([(0, 3000, 0.1, 300), (0, 500, 0.1, 20)] * 20)
+        all_, _ = passes([(0, 3000, 0.1, 300), (0, 12000, 0.1, 11000)])
+        assert k == 8 and all_ == 3 * few > 0
+    finally:
+        F.set_tuning(31, 8)
