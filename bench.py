@@ -106,7 +106,7 @@ def parse():
                     help="skip the batched and served forms")
     ap.add_argument("--workload", default="all",
                     choices=["all", "batched", "long", "two_lengths"],
-                    help="long: only the CTA-per-pair class (profiling); "
+                    help="long: only pairs of one index class (profiling); "
                          "batched: only the persistent launch of the uneven "
                          "batch (for profiling); two_lengths: only the "
                          "two-length comparison of forms")
@@ -114,6 +114,9 @@ def parse():
                     help="arrival window of each offered load")
     ap.add_argument("--batched-pairs", type=int, default=2_000_000,
                     help="pairs of the uneven batch")
+    ap.add_argument("--details", default=DETAILS, metavar="FILE",
+                    help="file for the whole record, of which the printed "
+                         "line holds the short values")
     return ap.parse_args()
 
 
@@ -415,6 +418,42 @@ def run_reference(args):
     }
     print(json.dumps(line), flush=True)
     return 0
+
+
+# Longest value (as JSON) that the printed line carries of its own: the whole
+# record was some 26 KB, longer than what a caller keeps of a program's
+# output, and could not be read back.
+LINE_VALUE_CHARS = 800
+DETAILS = os.path.join(ROOT, "paper_1910_09020_gb300", "_build",
+                       "bench_details.json")
+
+
+def short_line(line: dict, details: str | None) -> dict:
+    """The record without its long values (of a long section its numbers);
+    `details` is the file that holds all of it."""
+    out = {}
+    for k, v in line.items():
+        if len(json.dumps(v)) > LINE_VALUE_CHARS and isinstance(v, dict):
+            v = {x: y for x, y in v.items()
+                 if isinstance(y, (bool, int, float))}
+        if v != {} and len(json.dumps(v)) <= LINE_VALUE_CHARS:
+            out[k] = v
+    if details:
+        out["details"] = os.path.relpath(details, ROOT)
+    return out
+
+
+def print_line(line: dict, path: str) -> None:
+    """One JSON line on stdout, the whole record in the file `path`."""
+    try:
+        os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+        with open(path, "w") as f:
+            json.dump(line, f)
+            f.write("\n")
+    except OSError as err:
+        print(f"bench: {path} not written: {err}", file=sys.stderr)
+        path = None
+    print(json.dumps(short_line(line, path)), flush=True)
 
 
 def config_dict(world: int, n_override: int | None = None) -> dict:
@@ -1060,6 +1099,8 @@ def run_serving(seconds: float, slots: int = 2, ipk=None) -> dict:
                 "bound": "alu" if t == t_alu else "xu",
                 "t_alu_s": t_alu, "t_xu_s": t_xu, "burst_s": dt,
                 "alu_ops_per_pair": alu, "frac": t / dt,
+                "model": "every row of the maze, of which the index "
+                         "evaluates only a few: no bound of it",
                 "sample": f"op model from the oracle on {k} pairs drawn "
                           f"uniformly from the pool ({t_o:.1f} s)"}
         loads = []
@@ -1447,7 +1488,7 @@ def run_ours(args):
         "accuracy": accuracy,
         **extras,
     }
-    print(json.dumps(line), flush=True)
+    print_line(line, args.details)
     F.close()
     if world > 1:
         import torch.distributed as dist
@@ -1485,11 +1526,10 @@ def run_two_lengths_only(args):
 
 
 def run_long_only(args):
-    """The CTA-per-pair class alone (profiling aid): 608 pairs of 20 kbp,
-    edit rate 5 %, E = 10 % of the length (2000; 126 row words per pair,
-    four CTAs per SM), the shape of the served form's long pairs.  Two
-    filter passes without graph replay, so that a profiler sees every
-    launch; the busy k_cw_cta launch is the fifth of that kernel."""
+    """One index class alone (profiling aid): 608 pairs of 20 kbp, edit rate
+    5 %, E = 10 % of the length (2000), the shape of the served form's long
+    pairs.  Two filter passes without graph replay, so that a profiler sees
+    every launch; the busy launches are those of k_cw_index<1>."""
     import torch
 
     from paper_1910_09020_gb300 import binding, synth
@@ -1509,7 +1549,7 @@ def run_long_only(args):
         times.append(time.perf_counter() - t0)
     o = obs.cpu().numpy()
     print(json.dumps({"workload": f"{n} pairs x {m} bp, E = {int(E[0])}, "
-                                  "edit rate 5 %, CTA-per-pair class",
+                                  "edit rate 5 %, k_cw_index<1>",
                       "ms": [round(1e3 * t, 3) for t in times],
                       "greedy_iterations": int(o.sum()),
                       "accepted": int(acc.sum().item())}), flush=True)
