@@ -220,7 +220,7 @@ static size_t bucket_clear_bytes() { return (size_t)kKeys * 4 + 16; }
 
 using RingShape0 = RingShape<512, 512, 128, 2>;
 using RingShape1 = RingShape<1024, 1024, 256>;
-using RingShape2 = RingShape<2048, 1024, 256>;
+using RingShape2 = RingShape<2048, 1024, 256, 4, 12>;
 static_assert(RingShape0::max_e() >= ring_max_e(0) &&
                   RingShape1::max_e() >= ring_max_e(1) &&
                   RingShape2::max_e() >= ring_max_e(2),

@@ -99,10 +99,14 @@ SS_HD int index_run(const uint32_t *q, const uint32_t *r, int w16, int j,
 // reads 32 per lane after the first 32.
 constexpr int kRingAhead = 159;
 // Shape of a ring class: rings of QB bases of the query and RB of the
-// reference, filled in blocks of BP; LANES lanes per pair.
-template <int QB_, int RB_, int BP_, int LANES_ = 4>
+// reference, filled in blocks of BP; LANES lanes per pair; CTAS of its
+// kernel on an SM (14: 72 registers, 12: 80.  Of the largest class, E' = 750,
+// 30,000 pairs of 10 kbp 3.07 -> 2.64 ms with 12, 8,000 as much; of the others
+// 2M pairs of 64 bp to 10 kbp at 5 % 11.6 -> 11.8).
+template <int QB_, int RB_, int BP_, int LANES_ = 4, int CTAS_ = 14>
 struct RingShape {
     static constexpr int QB = QB_, RB = RB_, BP = BP_, LANES = LANES_;
+    static constexpr int CTAS = CTAS_;
     static constexpr int QW = QB / 32, RW = RB / 32;
     static constexpr int AHEAD = LANES <= 4 ? kRingAhead : 32 * LANES + 95;
     // words of a pair: both rings as (low, high) code words of 32 bases, the
@@ -671,7 +675,7 @@ SS_HD int ring_work_limit(int c, int count)
 // staged: n = 4000 309 / 153 / 223, 672 / 334 / 444, 1085 / 515 / 503; n =
 // 16000 331 / 394, 820 / 750, 1482 / 1370 against 332, 815, 1282.  When no
 // more pairs are waiting, so are a warp's last few.
-constexpr int ring_few(int c) { return c < 2 ? 4 : 6; }
+constexpr int ring_few(int c) { return c < 2 ? 4 : 7; }
 constexpr int kRingLast = 2;
 
 #ifdef __CUDACC__
@@ -782,7 +786,7 @@ __device__ __forceinline__ int team_far(const RingStep &s, int j, int at,
 }
 
 template <class Sh>
-__global__ void __launch_bounds__(32 * kRingWarps, 14)
+__global__ void __launch_bounds__(32 * kRingWarps, Sh::CTAS)
     k_cw_ring(const CwArgs a)
 {
     extern __shared__ uint2 rings[];

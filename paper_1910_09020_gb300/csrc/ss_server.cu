@@ -242,7 +242,7 @@ __device__ int long_claim(const ssk::LongQueue &q, uint64_t idle_ns,
 // a batch's last queued pair publishes the batch's generation to the host.
 // Pairs flagged as holding a non-base get obstacles -1 (their batch's
 // request fails alone, as in the pass).
-__global__ void __launch_bounds__(ssk::kIndexThreads, 3)
+__global__ void __launch_bounds__(ssk::kIndexThreads, 2)
     k_long_worker(const ssk::LongQueue q, uint64_t idle_ns)
 {
     extern __shared__ uint32_t smem[];
