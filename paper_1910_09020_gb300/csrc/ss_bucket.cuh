@@ -6,8 +6,8 @@
 // no Q base at all, so they are all obstacles and never bound the longest
 // run; the count limit still uses E):
 //   * RW classes: E' <= 31, thread per pair, E' <= EMAX in {1, 3, 7, 15, 31}
-//   * ring classes: E' <= 816, a team of 2 or 4 lanes per pair (ss_cws.cuh),
-//     by E'
+//   * ring classes: E' <= 816, a team of 2 or 4 lanes or (few pairs,
+//     repeats) a warp per pair (ss_cws.cuh), by E'
 //   * index classes: E' <= 10016, CTA per pair (ss_cwx.cuh), by E'
 //   * CTA classes: larger E', CTA per pair (ss_cw.cuh), by m bound
 // Within a class pairs are ordered by length, longest first (quarter-octave
@@ -215,9 +215,9 @@ struct LongQueue {
 constexpr int kLongRing = 1 << 18;   // entries (a power of two)
 constexpr int kLongBatches = 64;     // descriptors
 // Worker shape: one CTA per SM, routing a pair at a time with an index of up
-// to 98 KB (a pair of 100 kbp at E = 10^4), so that more than half of the
-// SM's shared memory stays free for the batches' own kernels (without room
-// beside the worker they waited for it to leave).
+// to 98 KB (a pair of 100 kbp at E = 10^4; above that all rows in 35 KB), so
+// that more than half of the SM's shared memory stays free for the batches'
+// own kernels (without room beside the worker they waited for it to leave).
 constexpr int kLongCtasPerSm = 1;
 
 // Whether the queue takes the pairs of class cls: the index and the CTA

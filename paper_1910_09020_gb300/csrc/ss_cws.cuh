@@ -388,6 +388,14 @@ SS_HD int warp_shfl(int v, int lane)
     return v;
 #endif
 }
+SS_HD int popc32(uint32_t x)
+{
+#ifdef __CUDA_ARCH__
+    return __popc(x);
+#else
+    return __builtin_popcount(x);
+#endif
+}
 SS_HD int warp_max(int v)
 {
 #ifdef __CUDA_ARCH__

@@ -41,15 +41,6 @@ SS_HD int ffs32(uint32_t x)
 #endif
 }
 
-SS_HD int popc32(uint32_t x)
-{
-#ifdef __CUDA_ARCH__
-    return __popc(x);
-#else
-    return __builtin_popcount(x);
-#endif
-}
-
 SS_HD int imax(int a, int b) { return a > b ? a : b; }
 SS_HD int imin(int a, int b) { return a < b ? a : b; }
 
